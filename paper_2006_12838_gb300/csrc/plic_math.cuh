@@ -138,18 +138,12 @@ template <> struct Fm<double> {
     static __device__ __forceinline__ int ilogb_(T w) { return ilogb(w); }
 };
 
-// Closed-form constants (Sec. 2.3, Eqs. 13-22; Sec. 2.4).  The two_* values are
-// the factor 2 of Eq. 11 folded into a3, b3, a4, b4 (the FP32 paired solver).
+// Closed-form constants (Sec. 2.3, Eqs. 13-22; Sec. 2.4).
 template <typename T> struct Kc {
     static constexpr T cbrt54 = (T)3.7797631496846195;             // 54^(1/3)       (a3 / n1 n2)
     static constexpr T inv_cbrt432 = (T)0.13228342099734996;       // 1 / 432^(1/3)  (b3)
     static constexpr T inv_cbrt864 = (T)0.10499342082457276;       // 1 / 864^(1/3)  (a4 / t4)
     static constexpr T inv_cbrt3456 = (T)0.066141710498674978;     // 1 / 3456^(1/3) (b4)
-    static constexpr T two_cbrt54 = (T)7.559526299369239;          // 2 * 54^(1/3)
-    static constexpr T two_over_cbrt432 = (T)0.26456684199469993;  // 2 / 432^(1/3)
-    static constexpr T two_over_cbrt864 = (T)0.20998684164914555;  // 2 / 864^(1/3)
-    static constexpr T two_over_cbrt3456 = (T)0.13228342099734997; // 2 / 3456^(1/3)
-    static constexpr T inv_sqrt12 = (T)0.28867513459481287;        // 1 / sqrt(12)
     static constexpr T pi_6 = (T)0.52359877559829887;              // pi / 6
     static constexpr T four_pi = (T)12.566370614359173;            // 4 pi
     static constexpr T third = (T)0.33333333333333333;

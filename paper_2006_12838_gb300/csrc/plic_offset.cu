@@ -260,50 +260,92 @@ k_plic_offset_compact(const T* __restrict__ nx, const T* __restrict__ ny, const 
     count_invalid(bad, invalid);
 }
 
-// The optimised SZ solution in FP32 (the paper's recommended solver, Sec.
-// 2.5) on paired FP32 instructions: each thread takes 4 cells per step as two
-// pairs.  Tail and unaligned cells go through the same pair code with the
-// cell duplicated in both lanes, so every cell sees identical arithmetic.
+// The optimised SZ, Kawano's SZ and the analytic solution in FP32 on paired
+// FP32 instructions: each thread takes 4 cells per step as two pairs, so every
+// cell sees identical arithmetic wherever it lies.  VEC (every array on a
+// 16-byte boundary): consecutive cells through one 16-byte load per array.
+// Otherwise (an odd row of a (3, n) tensor, a slice): cells 256 apart, each
+// array read in whole 128-byte lines of one warp, four loads per array in
+// flight.  The cells left over (n mod 4, n mod 1024) take one lane each, the cell in
+// both lanes of the pair; all unaligned cells that way took 88 us for 10 M cells
+// of the analytic solution, 39 us this way.
 // With ROUNDTRIP the forward volume of each stored d0 is written to vrt in
 // the same pass (plic_offset_roundtrip); COUNT (an invalid-cell counter was
 // given) keeps the per-cell count of invalid inputs, which otherwise costs
 // instructions for nothing.
-template <int METHOD, bool POLISH, bool ROUNDTRIP, bool COUNT>
-__global__ void __launch_bounds__(256)
+// Bound: HBM (20 B per cell, 24 with the round trip).  With the arcsine, the
+// sine and a Newton step on Eq. 10 in d these kernels were issue bound (131
+// instructions per cell in the round trip); with the depressed cubic
+// (p2::centre_distance), 2^26 cells: optimised SZ 265 -> 205 us, analytic
+// 320 -> 200 us (0.985 of the copy rate); round trip of 2^28 cells 1240 ->
+// 1000 us (0.945).  Residency of these two: five blocks per SM (48 registers)
+// without and four (64 registers) with the round trip is the fastest measured
+// (205 against 212 us at the compiler's 51 registers, 995 against 1004 us at 56).
+constexpr int pair_blocks(int method, bool roundtrip) {
+    return method == M_SZ_ORIG ? 0 : roundtrip ? 4 : 5;
+}
+
+template <int METHOD, bool POLISH, bool ROUNDTRIP, bool COUNT, bool VEC>
+__global__ void __launch_bounds__(256, pair_blocks(METHOD, ROUNDTRIP))
 k_plic_offset_pair(const float* __restrict__ nx, const float* __restrict__ ny,
                    const float* __restrict__ nz, const float* __restrict__ V0,
-                   float* __restrict__ d0, int64_t n, int vec_ok,
+                   float* __restrict__ d0, int64_t n, int /* vec_ok: VEC */,
                    unsigned long long* invalid, float* __restrict__ vrt) {
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int bad[2] = {0, 0}, bad1[2] = {0, 0};           // per lane of the pair; bad1: a cell in both lanes
+    float2 w0, w1;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int bad = 0;
-    const int64_t nvec = vec_ok ? n / 4 : 0;
-    for (int64_t i = tid; i < nvec; i += stride) {
-        const float4 a = __ldcs(reinterpret_cast<const float4*>(nx) + i);
-        const float4 b = __ldcs(reinterpret_cast<const float4*>(ny) + i);
-        const float4 c = __ldcs(reinterpret_cast<const float4*>(nz) + i);
-        const float4 v = __ldcs(reinterpret_cast<const float4*>(V0) + i);
-        float2 w0, w1;
-        const float2 r0 = p2::offset_pair<METHOD, POLISH, ROUNDTRIP, COUNT>(
-            make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y), make_float2(v.x, v.y),
-            bad, &w0);
-        const float2 r1 = p2::offset_pair<METHOD, POLISH, ROUNDTRIP, COUNT>(
-            make_float2(a.z, a.w), make_float2(b.z, b.w), make_float2(c.z, c.w), make_float2(v.z, v.w),
-            bad, &w1);
-        __stcs(reinterpret_cast<float4*>(d0) + i, make_float4(r0.x, r0.y, r1.x, r1.y));
-        if (ROUNDTRIP) __stcs(reinterpret_cast<float4*>(vrt) + i, make_float4(w0.x, w0.y, w1.x, w1.y));
+    int64_t tail;                                    // the cells from here on go one at a time
+    if constexpr (VEC) {
+        const int64_t nvec = n / 4;
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += stride) {
+            const float4 a = __ldcs(reinterpret_cast<const float4*>(nx) + i);
+            const float4 b = __ldcs(reinterpret_cast<const float4*>(ny) + i);
+            const float4 c = __ldcs(reinterpret_cast<const float4*>(nz) + i);
+            const float4 v = __ldcs(reinterpret_cast<const float4*>(V0) + i);
+            const float2 r0 = p2::offset_pair<METHOD, POLISH, ROUNDTRIP, COUNT>(
+                make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y), make_float2(v.x, v.y),
+                bad, &w0);
+            const float2 r1 = p2::offset_pair<METHOD, POLISH, ROUNDTRIP, COUNT>(
+                make_float2(a.z, a.w), make_float2(b.z, b.w), make_float2(c.z, c.w), make_float2(v.z, v.w),
+                bad, &w1);
+            __stcs(reinterpret_cast<float4*>(d0) + i, make_float4(r0.x, r0.y, r1.x, r1.y));
+            if (ROUNDTRIP) __stcs(reinterpret_cast<float4*>(vrt) + i, make_float4(w0.x, w0.y, w1.x, w1.y));
+        }
+        tail = nvec * 4;
+    } else {
+        tail = n & ~(int64_t)1023;
+        for (int64_t i0 = (int64_t)blockIdx.x * 1024; i0 < tail; i0 += 4 * stride) {
+            const int64_t i = i0 + threadIdx.x;
+            float a[4], b[4], c[4], v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                a[j] = __ldcs(nx + i + 256 * j);
+                b[j] = __ldcs(ny + i + 256 * j);
+                c[j] = __ldcs(nz + i + 256 * j);
+                v[j] = __ldcs(V0 + i + 256 * j);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; j += 2) {
+                const float2 r = p2::offset_pair<METHOD, POLISH, ROUNDTRIP, COUNT>(
+                    make_float2(a[j], a[j + 1]), make_float2(b[j], b[j + 1]), make_float2(c[j], c[j + 1]),
+                    make_float2(v[j], v[j + 1]), bad, &w0);
+                __stcs(d0 + i + 256 * j, r.x);
+                __stcs(d0 + i + 256 * (j + 1), r.y);
+                if (ROUNDTRIP) {
+                    __stcs(vrt + i + 256 * j, w0.x);
+                    __stcs(vrt + i + 256 * (j + 1), w0.y);
+                }
+            }
+        }
     }
-    for (int64_t i = nvec * 4 + tid; i < n; i += stride) {
-        int bad2 = 0;
-        float2 w;
+    for (int64_t i = tail + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const float2 r = p2::offset_pair<METHOD, POLISH, ROUNDTRIP, COUNT>(
             make_float2(nx[i], nx[i]), make_float2(ny[i], ny[i]), make_float2(nz[i], nz[i]),
-            make_float2(V0[i], V0[i]), bad2, &w);
-        bad += bad2 >> 1;
+            make_float2(V0[i], V0[i]), bad1, &w0);
         d0[i] = r.x;
-        if (ROUNDTRIP) vrt[i] = w.x;
+        if (ROUNDTRIP) vrt[i] = w0.x;
     }
-    if (COUNT) count_invalid(bad, invalid);
+    if (COUNT) count_invalid(bad[0] + bad[1] + bad1[0], invalid);
 }
 
 // PLIC_FP64_REFINED: double in/out, FP32 solve + two FP64 Newton steps.
@@ -364,21 +406,28 @@ static const void* pick(plic_precision p, bool faithful) {
                   : (faithful ? kptr<METHOD, float, false, true>() : kptr<METHOD, float, false, false>());
 }
 
-// The paired FP32 kernels (optimised SZ, analytic); *fused is set when the
-// round-trip volume comes out of the same kernel.
-template <int METHOD, bool COUNT>
-static const void* pick_pair_c(bool polish, bool roundtrip) {
-    if (polish)
-        return roundtrip ? reinterpret_cast<const void*>(&k_plic_offset_pair<METHOD, true, true, COUNT>)
-                         : reinterpret_cast<const void*>(&k_plic_offset_pair<METHOD, true, false, COUNT>);
-    return roundtrip ? reinterpret_cast<const void*>(&k_plic_offset_pair<METHOD, false, true, COUNT>)
-                     : reinterpret_cast<const void*>(&k_plic_offset_pair<METHOD, false, false, COUNT>);
+// The paired FP32 kernels (optimised SZ, Kawano's SZ, analytic); *fused is set
+// when the round-trip volume comes out of the same kernel.  The optimised SZ
+// and the analytic root end with their Newton step in either precision, so
+// FP32 and FP32_POLISHED are one kernel there.
+template <int METHOD, bool POLISH, bool VEC>
+static const void* pick_pair_k(bool roundtrip, bool count) {
+    if (roundtrip)
+        return count ? reinterpret_cast<const void*>(&k_plic_offset_pair<METHOD, POLISH, true, true, VEC>)
+                     : reinterpret_cast<const void*>(&k_plic_offset_pair<METHOD, POLISH, true, false, VEC>);
+    return count ? reinterpret_cast<const void*>(&k_plic_offset_pair<METHOD, POLISH, false, true, VEC>)
+                 : reinterpret_cast<const void*>(&k_plic_offset_pair<METHOD, POLISH, false, false, VEC>);
 }
 
 template <int METHOD>
-static const void* pick_pair(bool polish, bool roundtrip, bool count, bool* fused) {
+static const void* pick_pair(bool polish, bool roundtrip, bool count, bool vec, bool* fused) {
     *fused = roundtrip;
-    return count ? pick_pair_c<METHOD, true>(polish, roundtrip) : pick_pair_c<METHOD, false>(polish, roundtrip);
+    constexpr bool ONE = METHOD != M_SZ_ORIG;
+    if (polish || ONE)
+        return vec ? pick_pair_k<METHOD, true, true>(roundtrip, count)
+                   : pick_pair_k<METHOD, true, false>(roundtrip, count);
+    return vec ? pick_pair_k<METHOD, ONE, true>(roundtrip, count)
+               : pick_pair_k<METHOD, ONE, false>(roundtrip, count);
 }
 
 static plic_status offset_entry(const void* nx, const void* ny, const void* nz, const void* V0,
@@ -401,21 +450,22 @@ static plic_status offset_entry(const void* nx, const void* ny, const void* nz, 
     const int vec_ok = aligned(nx, 16) && aligned(ny, 16) && aligned(nz, 16) && aligned(V0, 16) &&
                        aligned(d0, 16) && (!vrt || aligned(vrt, 16));
     const bool faithful = (flags & PLIC_FLAG_FAITHFUL) != 0;
+    const bool pair = !dbl && !faithful && (m == PLIC_ANALYTIC || m == PLIC_SZ_ORIG || m == PLIC_SZ_OPT);
     const void* k = nullptr;
     switch (m) {
         case PLIC_ANALYTIC:
-            k = (!dbl && !faithful) ? pick_pair<M_ANALYTIC>(p == PLIC_FP32_POLISHED, vrt != nullptr,
-                                                            d_invalid_count != nullptr, fused)
+            k = pair ? pick_pair<M_ANALYTIC>(p == PLIC_FP32_POLISHED, vrt != nullptr,
+                                                            d_invalid_count != nullptr, vec_ok != 0, fused)
                                     : pick<M_ANALYTIC>(p, faithful);
             break;
         case PLIC_SZ_ORIG:
-            k = (!dbl && !faithful) ? pick_pair<M_SZ_ORIG>(p == PLIC_FP32_POLISHED, vrt != nullptr,
-                                                           d_invalid_count != nullptr, fused)
+            k = pair ? pick_pair<M_SZ_ORIG>(p == PLIC_FP32_POLISHED, vrt != nullptr,
+                                                           d_invalid_count != nullptr, vec_ok != 0, fused)
                                     : pick<M_SZ_ORIG>(p, faithful);
             break;
         case PLIC_SZ_OPT:
-            k = (!dbl && !faithful) ? pick_pair<M_SZ_OPT>(p == PLIC_FP32_POLISHED, vrt != nullptr,
-                                                          d_invalid_count != nullptr, fused)
+            k = pair ? pick_pair<M_SZ_OPT>(p == PLIC_FP32_POLISHED, vrt != nullptr,
+                                                          d_invalid_count != nullptr, vec_ok != 0, fused)
                                     : pick<M_SZ_OPT>(p, faithful);
             break;
         case PLIC_NEWTON: k = pick<M_NEWTON>(p, faithful); break;
@@ -423,7 +473,8 @@ static plic_status offset_entry(const void* nx, const void* ny, const void* nz, 
     }
     const int threads = 256;
     const int W = dbl ? 2 : 4;
-    const int64_t work = vec_ok ? (n + W - 1) / W : n;
+    // 4 cells per thread also where the paired kernels read unaligned arrays
+    const int64_t work = vec_ok || pair ? (n + W - 1) / W : n;
     const int grid = stream_grid(k, threads, work);
     unsigned long long* inv = reinterpret_cast<unsigned long long*>(d_invalid_count);
     void* args[] = {(void*)&nx, (void*)&ny, (void*)&nz, (void*)&V0, (void*)&d0,

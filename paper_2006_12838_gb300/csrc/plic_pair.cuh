@@ -4,12 +4,11 @@
 // issues two FP32 operations).  Comparisons, selects and
 // MUFU operations stay per component.
 //
-// The arithmetic is that of solve_sz_opt_default<float> + polish (see
-// plic_solvers.cuh): the division-free case tests, the cancellation-free
-// arcsine argument, all cases evaluated and selected, and, for the polished
-// precision, one Newton step on the cubic of Eq. 10 for the cells whose root
-// came from the trigonometric formula (cases 3/4; the closed forms of cases
-// 1, 2, 5 are already accurate to a few ulp).
+// All cases are evaluated and selected.  The optimised SZ and the analytic
+// solution form the root of cases (3)/(4) from the depressed cubic
+// (centre_distance) with a Newton step in both FP32 precisions; Kawano's form
+// keeps its arccosine, and for the polished precision one Newton step on the
+// cubic of Eq. 10 (the closed forms of cases 1, 2, 5 are accurate to a few ulp).
 #pragma once
 #include "plic_solvers.cuh"
 
@@ -46,15 +45,6 @@ __device__ __forceinline__ f2 cbrt_(f2 x) {
     x = add(x, mk(1e-30f));
     return make_float2(Fm<float>::exp2f_approx(Fm<float>::__log2f_approx(x.x) * (1.0f / 3.0f)),
                        Fm<float>::exp2f_approx(Fm<float>::__log2f_approx(x.y) * (1.0f / 3.0f)));
-}
-
-// The same cube root with one Newton step (relative error at FP32 rounding):
-// for the analytic solution, whose trigonometric root scales with u^(1/2).
-__device__ __forceinline__ f2 cbrt_nr(f2 x) {
-    const f2 r = cbrt_(x);
-    const f2 r2 = mul(r, r);
-    const f2 res = fma(r2, r, make_float2(-x.x - 1e-30f, -x.y - 1e-30f));     // r^3 - x
-    return fma(make_float2(-res.x, -res.y), rcp(mul(mk(3.0f), r2)), r);
 }
 
 // sqrt of x >= 0 as x rsqrt(x) with 1e-30 added (no zero branch).  Both
@@ -104,52 +94,64 @@ __device__ __forceinline__ f2 polish34(f2 d, f2 V6, f2 n1, f2 n2, f2 n3) {
     return sub(d, mul(g, rcp(gp)));
 }
 
-// Reduced optimised-SZ solution for two cells (L1-normalised m1 <= m2 <= m3,
-// reduced volume V).  The trigonometric root of cases (3)/(4) is formed (and,
-// with POLISH, given its Newton step) first; the closed forms of cases (2),
-// (1) and (5) then replace it, each select right after its test, so that no
-// case flag stays live across the long trigonometric chain.
-template <bool POLISH>
-__device__ __forceinline__ f2 sz_opt(f2 V, f2 n1, f2 n2, f2 n3) {
-    const f2 n12 = add(n1, n2), n3V = mul(n3, V);
-    const f2 n3V2 = add(n3V, n3V);
-    const f2 V6n2n3 = mul(mul(mk(6.0f), n2), n3V), sqn1 = mul(n1, n1);
-    const f2 n1n2 = mul(n1, n2);
-    // case (3) vs (4): 6 n1 n2 n3 V < n3^2 (3 n12 - n3) + n1^2 (n1 - 3 n3) + n2^2 (n2 - 3 n3)
-    f2 num3 = mul(mul(n3, n3), fma(mk(3.0f), n12, make_float2(-n3.x, -n3.y)));
-    num3 = fma(sqn1, fma(mk(-3.0f), n3, n1), num3);
-    num3 = fma(mul(n2, n2), fma(mk(-3.0f), n3, n2), num3);
-    const b2 n3small = lt(n3, n12);
-    const f2 V6n1n2n3 = mul(V6n2n3, n1);
-    const b2 v3lt = lt(V6n1n2n3, num3);
-    const b2 c3 = {!n3small.x || v3lt.x, !n3small.y || v3lt.y};
-    // arcsine argument without cancellation
-    const f2 q3 = mul(mul(mk(1.5f), n1n2), sub(n12, n3V2));
-    const f2 q4 = mul(mul(mul(mk(0.75f), n1n2), n3), fma(mk(-2.0f), V, mk(1.0f)));
-    const f2 d32 = sub(n3, n2);
-    const f2 t24 = mul(mk(0.25f), fma(n1, fma(mk(2.0f), add(n2, n3), make_float2(-n1.x, -n1.y)),
-                                     make_float2(-d32.x * d32.x, -d32.y * d32.y)));
-    const f2 q = sel(c3, q3, q4);
-    const f2 t2 = sel(c3, add(n1n2, n1n2), t24);
-    const f2 c = sel(c3, n12, mk(0.5f));
-    const f2 rt = rsqrt(t2);
-    const f2 t = mul(t2, rt);
-    f2 arg = mul(q, mul(rt, mul(rt, rt)));
-    arg = make_float2(fminf(arg.x, 1.0f), fminf(arg.y, 1.0f));
-    const f2 th = mul(mk(0.33333333333333333f), asin01(arg));
-    const f2 sn = make_float2(__sinf(th.x), __sinf(th.y));
-    f2 d = fma(mul(mk(-2.0f), t), sn, c);
-    if (POLISH) d = polish34(d, V6n1n2n3, n1, n2, n3);
-    // case (2) where 3 n2 (2 n3 V + n1 - n2) < n1^2, unless case (1) holds
-    const f2 t2a = mul(mul(mk(3.0f), n2), add(n3V2, sub(n1, n2)));
-    const f2 d2 = mul(mk(0.5f), add(n1, sqrtp(fma(mk(8.0f), mul(n2, n3V), mul(mk(-0.33333333333333333f), sqn1)))));
-    d = sel(lt(t2a, sqn1), d2, d);
-    // case (1) where 6 n2 n3 V < n1^2
-    const f2 d1 = cbrt_(V6n1n2n3);
-    d = sel(lt(V6n2n3, sqn1), d1, d);
-    // case (5) where n1 + n2 <= 2 n3 V
-    const f2 d5 = fma(mk(0.5f), n12, n3V);
-    return sel(le(n12, n3V2), d5, d);
+// The smaller positive root w of the depressed cubic w^3 - Q w + R = 0 of cases
+// (3)/(4), from nQ = -Q < 0 and R >= 0 (sz_opt below).  Viete's form is
+// w = 2 t sin(asin(a)/3) with t^2 = Q/3, a = R/(2 t^3); in these cases
+// a <= 0.8839, clear of the arcsine's singular end, so one odd polynomial (an
+// equal-ripple fit of 2 sin(asin(a)/3) on a <= 0.886, degree 9, within 8e-5)
+// stands for the arcsine, its half-angle reduction and the sine.  It is
+// evaluated in x = R Q^(-3/2), the powers of 3^(1/2) in t and a folded into
+// its coefficients.  One Newton step on the cubic (quadratic term: 9e-9 t) then
+// makes the root as accurate as Q and R are.
+__device__ __forceinline__ f2 depressed_root(f2 nQ, f2 R) {
+    const f2 rq = make_float2(rsqrtf(-nQ.x), rsqrtf(-nQ.y));
+    const f2 x = mul(mul(R, rq), mul(rq, rq));
+    const f2 z = mul(x, x);
+    f2 p = fma(mk(-704.3350219726562f), z, mk(107.44769287109375f));
+    p = fma(p, z, mk(-10.902824401855469f));
+    p = fma(p, z, mk(-0.8008332848548889f));
+    p = fma(p, z, mk(-1.001369833946228f));
+    const f2 w = mul(mul(nQ, rq), mul(x, p));
+    const f2 q = fma(w, w, nQ);                                   // w^2 - Q
+    const f2 f = fma(w, q, R), df = fma(add(w, w), w, q);         // 3 w^2 - Q < 0
+    return sub(w, mul(f, rcp(df)));
+}
+
+// The optimised SZ and the analytic solution for two cells in the reduced
+// space (n1 <= n2 <= n3, reduced volume V), as the distance s = L/2 - d of the
+// plane from the cell's centre (L = n1 + n2 + n3; `half` = L/2, `twice` = 2 L:
+// constants in the L1 units of SZ).  With p = n1 n2 and B = n1 + n2 - 2 n3 V,
+// Eq. 10 about its inflection point is the depressed cubic w^3 - Q w + R = 0:
+//   case (3), w = n1 + n2 - d: Q = 6 p,  R = 3 p B;
+//   case (4), w = L/2 - d = s: Q = 3/4 (n1 (2 L - 3 n1) - (n3 - n2)^2),
+//                              R = 3 p n3 (1/2 - V);
+// the trigonometric roots of both solutions (Eq. 11 with Eqs. 12-22, and the
+// merged arcsine of Sec. 2.4) are its smaller positive root.  The other cases
+// are s = n3 (1/2 - V) (5), s = L/2 - n1/2 - (2 n2 n3 V - n1^2/12)^(1/2) (2)
+// and s = L/2 - (6 p n3 V)^(1/3) (1).  Tests: (5) B <= 0; (1) or (2)
+// 3 n2 (2 n1 - B) < n1^2, of these (1) where 6 n2 n3 V < n1^2; (4) where the
+// case-(3) cubic is negative at d = n3 (g = n1 + n2 - n3 > 0):
+// g^3 + 3 p (B - 2 g) < 0.  The tests use the B of the root, so a root is only
+// taken with a <= 0.884.
+__device__ __forceinline__ f2 centre_distance(f2 V, f2 n1, f2 n2, f2 n3, f2 half, f2 twice) {
+    const f2 n12 = add(n1, n2), p3 = mul(mul(mk(3.0f), n1), n2);
+    const f2 h = mul(n3, V), B = fma(mk(-2.0f), h, n12);
+    const f2 s5 = mul(n3, sub(mk(0.5f), V));
+    // cases (2) and (1)
+    const f2 k = mul(n2, h), k6 = mul(mk(6.0f), k), sq1 = mul(n1, n1);
+    const f2 d2 = fma(mk(0.5f), n1, sqrtp(fma(mk(2.0f), k, mul(mk(-0.083333333333333333f), sq1))));
+    const f2 d12 = sel(lt(k6, sq1), cbrt_(mul(k6, n1)), d2);
+    // case (3) or (4)
+    const f2 g = sub(n12, n3);
+    const f2 t4 = fma(mul(g, g), g, mul(p3, fma(mk(-2.0f), g, B)));
+    const b2 c4 = {g.x > 0.0f && t4.x < 0.0f, g.y > 0.0f && t4.y < 0.0f};
+    const f2 e = fma(n1, fma(mk(-3.0f), n1, twice), mul(sub(n3, n2), sub(n2, n3)));
+    // 1e-36 keeps the reciprocal square root finite at n1 = 0 (case (2) or (5))
+    const f2 nQ = sel(c4, mul(mk(-0.75f), e), fma(mk(-2.0f), p3, mk(-1e-36f)));
+    const f2 w = depressed_root(nQ, mul(p3, sel(c4, s5, B)));
+    f2 s = add(w, sel(c4, mk(0.0f), sub(half, n12)));
+    s = sel(lt(mul(mul(mk(3.0f), n2), sub(add(n1, n1), B)), sq1), sub(half, d12), s);
+    return sel(le(B, mk(0.0f)), s5, s);
 }
 
 // Kawano's Scardovelli-Zaleski solution (Sec. 2.4) for two cells, in the
@@ -205,75 +207,6 @@ __device__ __forceinline__ f2 sz_orig(f2 w, f2 m1, f2 m2, f2 m3) {
     return sel(lt(w, vb1), d1, d);
 }
 
-// The paper's analytic solution (Sec. 2.3, Eq. 25 with the tests of Eq. 24)
-// for two cells, in the reduced space of the unit normal (n1 <= n2 <= n3,
-// |n| = 1, V the reduced volume).  As in sz_opt: case (3) or (4) is decided
-// first from the volume at d = n3 (the test d3 <= n3 of the paper, made before
-// forming d3), so that one trigonometric root f(x, y, a, b, c) is evaluated
-// with the coefficients of that case; with u^3 = x^2 + y^2 the arctangent
-// atan(y/x) (x >= 0 here) is asin(y/u^(3/2)).  With POLISH the root gets
-// one Newton step; then the closed forms of cases (2), (1), (5) replace it
-// where their tests hold.
-template <bool POLISH>
-__device__ __forceinline__ f2 analytic(f2 V, f2 n1, f2 n2, f2 n3) {
-    typedef Kc<float> K;
-    const f2 n12 = add(n1, n2), n3V = mul(n3, V);
-    const f2 n3V2 = add(n3V, n3V);
-    const f2 V6n2n3 = mul(mul(mk(6.0f), n2), n3V), sqn1 = mul(n1, n1);
-    const f2 n1n2 = mul(n1, n2);
-    // case (3) vs (4): 6 n1 n2 n3 V < n3^2 (3 n12 - n3) + n1^2 (n1 - 3 n3) + n2^2 (n2 - 3 n3)
-    f2 num3 = mul(mul(n3, n3), fma(mk(3.0f), n12, make_float2(-n3.x, -n3.y)));
-    num3 = fma(sqn1, fma(mk(-3.0f), n3, n1), num3);
-    num3 = fma(mul(n2, n2), fma(mk(-3.0f), n3, n2), num3);
-    const b2 n3small = lt(n3, n12);
-    const f2 V6n1n2n3 = mul(V6n2n3, n1);
-    const b2 v3lt = lt(V6n1n2n3, num3);
-    const b2 c3 = {!n3small.x || v3lt.x, !n3small.y || v3lt.y};
-    // coefficients: case (3) x3 = 81 n1 n2 (n12 - 2 n3 V), y3^2 = 23328 (n1 n2)^3 - x3^2;
-    // case (4) t4 = 9 (n12 + n3)^2 - 18, x4 = n1 n2 n3 (324 - 648 V), y4^2 = 4 t4^3 - x4^2
-    const f2 x3 = mul(mul(mk(81.0f), n1n2), sub(n12, n3V2));
-    const f2 p3 = mul(mul(n1n2, n1n2), n1n2);
-    const f2 y3 = fma(mk(23328.0f), p3, make_float2(-x3.x * x3.x, -x3.y * x3.y));
-    const f2 s4 = add(n12, n3);
-    const f2 t4 = fma(mk(9.0f), mul(s4, s4), mk(-18.0f));
-    f2 x4 = mul(mul(n1n2, n3), fma(mk(-648.0f), V, mk(324.0f)));
-    x4 = make_float2(fmaxf(x4.x, 1.17549435e-38f), fmaxf(x4.y, 1.17549435e-38f));
-    const f2 y4 = fma(mul(mk(4.0f), t4), mul(t4, t4), make_float2(-x4.x * x4.x, -x4.y * x4.y));
-    const f2 x = sel(c3, x3, x4);
-    const f2 ysq = fmax0(sel(c3, y3, y4));
-    const f2 a = sel(c3, mul(mk(K::two_cbrt54), n1n2), mul(mk(K::two_over_cbrt864), t4));
-    const f2 b = sel(c3, mk(K::two_over_cbrt432), mk(K::two_over_cbrt3456));
-    const f2 c = sel(c3, n12, mul(mk(0.5f), s4));
-    const f2 q = fma(x, x, ysq);                                     // u^3
-    const f2 u = cbrt_nr(q);
-    // atan(y/x) from sine and cosine: the arcsine of the smaller of the two
-    // (<= 1/sqrt 2), reflected about pi/4 where y > x -- the arcsine of a
-    // sine near 1 would lose half the digits (x -> 0 near V = 1/2 in case (4)
-    // and near the case-(5) boundary in case (3))
-    const f2 rq = rsqrt(add(q, mk(1e-30f)));
-    const f2 sv = mul(sqrtp(ysq), rq), cv = mul(x, rq);
-    const b2 refl = lt(cv, sv);
-    const f2 am = sel(refl, cv, sv);
-    const f2 as = asin01(make_float2(fminf(am.x, 1.0f), fminf(am.y, 1.0f)));
-    const f2 th = mul(mk(0.33333333333333333f), sel(refl, sub(mk(1.5707963267948966f), as), as));
-    const f2 ang = sub(mk(K::pi_6), th);
-    const f2 sn = make_float2(__sinf(ang.x), __sinf(ang.y));
-    f2 d = fma(mul(fma(b, u, a), rsqrt(u)), make_float2(-sn.x, -sn.y), c);
-    if (POLISH) d = polish34(d, V6n1n2n3, n1, n2, n3);
-    // case (2) where 3 n2 (2 n3 V + n1 - n2) < n1^2, unless case (1) holds
-    const f2 t2a = mul(mul(mk(3.0f), n2), add(n3V2, sub(n1, n2)));
-    const f2 d2 = fma(mk(0.5f), n1, mul(mk(K::inv_sqrt12),
-                                        sqrtp(fma(mk(24.0f), mul(n2, n3V), make_float2(-sqn1.x, -sqn1.y)))));
-    d = sel(lt(t2a, sqn1), d2, d);
-    // case (1) where 6 n2 n3 V < n1^2 (the plain cube root: d1 <= n1, so its
-    // relative error leaves an absolute one below 2e-7, as in sz_opt)
-    const f2 d1 = cbrt_(V6n1n2n3);
-    d = sel(lt(V6n2n3, sqn1), d1, d);
-    // case (5) where n1 + n2 <= 2 n3 V
-    const f2 d5 = fma(mk(0.5f), n12, n3V);
-    return sel(le(n12, n3V2), d5, d);
-}
-
 // Forward volume (Eq. 10) of two cells at their offsets d0, in the cell's
 // L1-normalised reduced space (m1 <= m2 <= m3, m1 + m2 + m3 = 1; Eq. 10 is
 // homogeneous of degree 0 in (d, n)), il = 1/L:
@@ -291,15 +224,13 @@ __device__ __forceinline__ f2 volume_reduced(f2 d0, f2 il, f2 m1, f2 m2, f2 m3) 
     const f2 m12 = add(m1, m2);
     const f2 v5 = mul(fma(mk(-0.5f), m12, d), rcp(m3));
     const f2 r1 = rcp(m1), r23 = rcp(mul(mk(6.0f), mul(m2, m3)));
-    const f2 v1 = mul(mul(mul(d, d), d), mul(r1, r23));
     const f2 inv1 = make_float2(fminf(r1.x, 3.40282347e38f), fminf(r1.y, 3.40282347e38f));
     const f2 e2 = fmax0(sub(d, m2)), e3 = fmax0(sub(d, m3));
     const f2 cub = fma(mul(e2, e2), e2, mul(mul(e3, e3), e3));
     f2 num = fma(mul(mk(3.0f), d), sub(d, m1), mul(m1, m1));
     num = fma(make_float2(-cub.x, -cub.y), inv1, num);
-    const f2 v24 = mul(num, r23);
-    f2 v = sel(lt(d, m1), v1, v24);
-    v = sel(le(m12, d), v5, v);
+    num = sel(lt(d, m1), mul(mul(mul(d, d), d), inv1), num);       // case (1)
+    const f2 v = sel(le(m12, d), v5, mul(num, r23));
     return make_float2(d0.x > 0.0f ? 1.0f - v.x : v.x, d0.y > 0.0f ? 1.0f - v.y : v.y);
 }
 
@@ -307,9 +238,9 @@ __device__ __forceinline__ f2 volume_reduced(f2 d0, f2 il, f2 m1, f2 m2, f2 m3) 
 // (METHOD = M_SZ_OPT, in L1 units), Kawano's SZ solution (M_SZ_ORIG, in L1
 // units) or the analytic solution (M_ANALYTIC, in the unit normal's units);
 // with ROUNDTRIP, also the forward volume of the returned d0 into *vrt; with
-// COUNT, invalid cells are added to `bad`.
+// COUNT, invalid cells are added to `bad` (one count per cell of the pair).
 template <int METHOD, bool POLISH, bool ROUNDTRIP = false, bool COUNT = true>
-__device__ __forceinline__ f2 offset_pair(f2 nx, f2 ny, f2 nz, f2 V0, int& bad,
+__device__ __forceinline__ f2 offset_pair(f2 nx, f2 ny, f2 nz, f2 V0, int (&bad)[2],
                                           f2* vrt = nullptr) {
     const f2 ax = make_float2(fabsf(nx.x), fabsf(nx.y));
     const f2 ay = make_float2(fabsf(ny.x), fabsf(ny.y));
@@ -323,19 +254,21 @@ __device__ __forceinline__ f2 offset_pair(f2 nx, f2 ny, f2 nz, f2 V0, int& bad,
     const f2 V = make_float2(fminf(V0.x, W.x), fminf(V0.y, W.y));
     const bool okx = V.x >= 0.0f && L.x > 0.0f && L.x <= 3.0f;
     const bool oky = V.y >= 0.0f && L.y > 0.0f && L.y <= 3.0f;
-    if (COUNT) bad += (int)!okx + (int)!oky;
+    if (COUNT) {
+        bad[0] += (int)!okx;
+        bad[1] += (int)!oky;
+    }
     const f2 il = rcp(L);
     const f2 m1 = mul(n1, il), m3 = mul(n3, il);
     const f2 m2 = fmax0(sub(mk(1.0f), add(m1, m3)));
     f2 h;
     if (METHOD == M_SZ_OPT) {
-        h = mul(L, sub(mk(0.5f), sz_opt<POLISH>(V, m1, m2, m3)));
+        h = mul(L, centre_distance(V, m1, m2, m3, mk(0.5f), mk(2.0f)));
     } else if (METHOD == M_SZ_ORIG) {
         h = mul(L, sub(mk(0.5f), sz_orig<POLISH>(V, m1, m2, m3)));
     } else {
         const f2 n2 = fmax0(sub(sub(L, n1), n3));
-        const f2 d = analytic<POLISH>(V, n1, n2, n3);
-        h = fma(mk(0.5f), L, make_float2(-d.x, -d.y));
+        h = centre_distance(V, n1, n2, n3, mul(mk(0.5f), L), add(L, L));
     }
     f2 r = make_float2(copysignf(h.x, V0.x - 0.5f), copysignf(h.y, V0.y - 0.5f));
     if (!okx) r.x = __int_as_float(0x7fffffff);

@@ -111,8 +111,8 @@ k_vof_curvature_nn(const float* __restrict__ phi, int nx, int ny, int nz,
             }
             float d0i[2];
             if (METHOD == M_SZ_OPT || METHOD == M_ANALYTIC) {
-                int bad = 0;
-                const p2::f2 r = p2::offset_pair<METHOD, true, false>(
+                int bad[2];                          // not counted
+                const p2::f2 r = p2::offset_pair<METHOD, true, false, false>(
                     make_float2(mx[0], mx[1]), make_float2(my[0], my[1]), make_float2(mz[0], mz[1]),
                     make_float2(v[0], v[1]), bad);
                 d0i[0] = r.x;
