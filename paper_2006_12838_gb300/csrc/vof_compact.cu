@@ -1,30 +1,33 @@
 // vof_compact.cu -- interface-cell compaction (Sec. 4.1, Eq. 33): the ordered
 // list of interior cells with 0 < phi < 1, and plic_workspace_bytes().
 //
-// Two or three launches, no atomics and no inter-block waiting, so the list
-// is in ascending cell order and identical run to run.  A tile is a run of
-// whole x-rows (about 8192 cells):
-//   1. k_compact_count : each block counts the interface cells of its tile and,
-//                        with room in the workspace, stores the tile's
-//                        interface bits (one word per 32 cells of a row);
-//                        k_compact_count_p2 does the same for 16-byte aligned
-//                        rows of 128 * 2^k cells with slot arithmetic in
-//                        shifts and masks.
-//   2. k_compact_scan  : one block turns the per-tile counts into exclusive
-//                        offsets (in place) and writes the total to *d_count;
-//                        only for fields of more than 4096 tiles (about 33 M
-//                        cells): below, pass 3 sums the counts of the tiles
-//                        before each block, and the warp of the last tile
-//                        writes the total.
-//   3. k_compact_emit  : one warp per tile writes the indices of the tile's
-//                        cells from the stored bits.  Without room for the bits
-//                        (rows shorter than 32 cells) or without a workspace
-//                        (the allocation-free entry), k_compact_write recounts
-//                        each row from the field and scans the row counts
-//                        itself.
-// HBM roofline: 4 B per field cell read once + 1/8 B per cell of bits written
-// and read back for the tiles holding interface cells, plus 4 B per interface
-// cell written.
+// Two launches, no atomics on global memory and no inter-block waiting, so the
+// list is in ascending cell order and identical run to run.  The field is
+// taken as one flat run of cells (the planes z = 0 and z = nz - 1 left out),
+// whatever its rows: a chunk is 32 lanes x 4 U cells, a tile CT_WARPS x K chunks.
+//   1. k_compact_count : reads the field once.  A warp first asks whether its
+//                        chunk holds any value in (0, 1) at all -- one fused
+//                        multiply-add v - v^2 and half a three-way maximum
+//                        per cell, one vote per chunk -- and goes on only
+//                        where it does (a quarter of the chunks of a field of
+//                        droplets): there it tests the cells exactly, drops
+//                        those on the field's boundary (the only place where
+//                        x, y and z are needed) and stores the chunk's bits, one
+//                        word per 32 cells.  Per tile it writes the count and a
+//                        mask of the chunks that hold cells, and per block of
+//                        S tiles the sum of their counts.
+//   2. k_compact_emit  : one warp per tile sums the counts before it and writes
+//                        the indices from the stored bits of the marked
+//                        chunks, or (no bits: the allocation-free entry) from
+//                        the field again, marked chunks only.
+// Bound: HBM, 4 B per field cell read once (+ 1/8 B of bits for marked chunks,
+// + 4 B per interface cell).  Times of the two passes (fields read from HBM),
+// against a row-wise pass that packed every cell's test into bits: 64^3 14.2 +
+// 5.6 -> 5.9 + 5.3 us; 301 x 203 x 257 (rows that are not whole 16-byte
+// vectors, read cell by cell before) 42.9 + 10.0 -> 13.7 + 6.7 us; 256^3 15.1 +
+// 6.2 -> 15.0 + 6.8 us (in L2, with the curvature after it: 29.0 -> 24.1 us);
+// 1 GiB 170.7 + 24.8 (with a scan launch between) -> 153.4 + 18.7 us, the
+// plain read being 149.
 #include <mutex>
 #include <stdio.h>
 
@@ -34,595 +37,407 @@ namespace plic {
 
 constexpr int CT_THREADS = 256;
 constexpr int CT_WARPS = CT_THREADS / 32;
-constexpr int CT_TILE = 8192;            // cells per tile (whole x-rows)
-constexpr int CT_MAX_ROWS = 4096;        // rows per tile at most (CT_TILE / 3 for nx >= 3)
-constexpr int CT_MAX_WORDS = 2048;       // ballot words per tile kept in shared memory
-constexpr int64_t CT_FUSED_SCAN_TILES = 4096;   // tiles up to which pass 3 does its own prefix sum
+// tiles or blocks of tiles whose counts the write pass sums in front of each block
+constexpr int64_t CT_MAX_SUPERS = 8192;
 
-// Rows (x-lines) per tile: as many whole rows as fit in CT_TILE cells.
-__host__ __device__ inline int tile_rows(int nx) {
-    const int r = nx > 0 ? CT_TILE / nx : 1;
-    return r < 1 ? 1 : (r > CT_MAX_ROWS ? CT_MAX_ROWS : r);
-}
+// How a field is cut: cells [base, base + cells) of the flat field (base a
+// multiple of 32 cells), tiles of `tile` cells, S tiles per block of pass 1.
+struct CompactPlan {
+    int64_t base, cells, tiles, supers;
+    int tile, S;
+};
 
-__device__ __forceinline__ bool iface(float v) { return v > 0.0f && v < 1.0f; }
-
-// Interface bits of one row, 32 cells per word (bit x % 32 of word x / 32),
-// with the boundary columns x = 0 and x = nx - 1 cleared; the caller has
-// checked the row's y and z.  `fn(word_index, bits)` is called by one lane per
-// word; returns the row's count in every lane.  With 16-byte aligned rows
-// (nx % 4 == 0) each lane loads 4 cells at once.
-template <typename F>
-__device__ __forceinline__ int row_bits(const float* __restrict__ row, int nx, bool vec, F fn) {
-    const int lane = threadIdx.x & 31;
-    int cnt = 0;
-    if (vec) {
-        for (int x0 = 0; x0 < nx; x0 += 128) {
-            const int x = x0 + 4 * lane;
-            unsigned m = 0u;
-            if (x < nx) {
-                const float4 v = __ldg(reinterpret_cast<const float4*>(row + x));
-                m = (unsigned)iface(v.x) | ((unsigned)iface(v.y) << 1) |
-                    ((unsigned)iface(v.z) << 2) | ((unsigned)iface(v.w) << 3);
-                if (x == 0) m &= ~1u;
-                if (x + 3 == nx - 1) m &= ~8u;
-            }
-            // gather the nibbles of 8 lanes into one 32-bit word
-            unsigned w = m << (4 * (lane & 7));
-            w |= __shfl_xor_sync(0xffffffffu, w, 1);
-            w |= __shfl_xor_sync(0xffffffffu, w, 2);
-            w |= __shfl_xor_sync(0xffffffffu, w, 4);
-            cnt += __popc(m);
-            if ((lane & 7) == 0 && x < nx) fn((x0 >> 5) + (lane >> 3), w);
-        }
-    } else {
-        for (int x0 = 0; x0 < nx; x0 += 32) {
-            const int x = x0 + lane;
-            const float v = x < nx ? __ldg(row + x) : 0.0f;
-            const unsigned b = __ballot_sync(0xffffffffu, x >= 1 && x <= nx - 2 && iface(v));
-            cnt += (b >> lane) & 1u;
-            if (lane == 0) fn(x0 >> 5, b);
-        }
-    }
-    return __reduce_add_sync(0xffffffffu, cnt);
+// Tile sizes: 8192 cells (16 loads of 16 bytes per lane in flight) where the
+// field gives every SM several blocks of it, smaller tiles below, where the
+// pass lasts as long as one block (64^3: 248 tiles of 1024 cells 5.9 us, 32 tiles
+// of 8192 14 us).  S grows once the write pass would have to sum more
+// than CT_MAX_SUPERS counts (above 67 M cells; one scan launch in between took
+// 11 us on 1 GiB).
+static CompactPlan compact_plan(int nx, int ny, int nz) {
+    CompactPlan p;
+    const int64_t nxy = (int64_t)nx * ny;
+    p.base = nxy & ~(int64_t)31;
+    p.cells = nxy * (nz - 1) - p.base;
+    p.tile = p.cells >= (int64_t)5 << 20 ? 8192 : p.cells >= (int64_t)1 << 20 ? 4096 : 1024;
+    p.tiles = (p.cells + p.tile - 1) / p.tile;
+    p.S = 1;
+    while ((p.tiles + p.S - 1) / p.S > CT_MAX_SUPERS) p.S *= 2;
+    p.supers = (p.tiles + p.S - 1) / p.S;
+    return p;
 }
 
 // The interface test 0 < phi < 1 on the float's bits: the positive floats
 // below 1.0f are exactly the bit patterns 1 .. 0x3F7FFFFF (zero, negative
-// values, 1.0f and above, infinities and NaNs all fall outside), so one
-// unsigned compare of u - 1 decides it.
-__device__ __forceinline__ bool iface_bits(unsigned u) { return u - 1u < 0x3F7FFFFFu; }
+// values, 1.0f and above, infinities and NaNs all fall outside).
+__device__ __forceinline__ bool iface_bits(float v) { return __float_as_uint(v) - 1u < 0x3F7FFFFFu; }
 
-// Vector path helpers: the 4-bit interface mask of the float4 at column x of
-// a row (boundary columns cleared), and the gather of the nibbles of 8 lanes
-// into the row's 32-bit word (x0 / 32 + lane / 8), stored by `fn`.
-__device__ __forceinline__ unsigned nib4(float4 v, int x, int nx) {
-    unsigned m = (unsigned)iface_bits(__float_as_uint(v.x)) |
-                 ((unsigned)iface_bits(__float_as_uint(v.y)) << 1) |
-                 ((unsigned)iface_bits(__float_as_uint(v.z)) << 2) |
-                 ((unsigned)iface_bits(__float_as_uint(v.w)) << 3);
-    if (x == 0) m &= ~1u;
-    if (x + 3 == nx - 1) m &= ~8u;
-    return x < nx ? m : 0u;
-}
+// Positive exactly for 0 < v < 1 (v - v^2 rounded once: its sign is that of
+// v (1 - v), and it does not underflow to 0, since v - v^2 >= 2^-149 there);
+// NaN for a NaN and for +inf - inf, which the maxima below skip.
+__device__ __forceinline__ float inside(float v) { return fmaf(-v, v, v); }
+__device__ __forceinline__ float max3(float a, float b, float c) { return fmaxf(fmaxf(a, b), c); }
 
-template <typename F>
-__device__ __forceinline__ void emit_nibbles(unsigned m, int x0, int nx, F fn) {
+// Division of 0 <= n < 2^31 by a divisor fixed per launch: with l =
+// ceil(log2 d) and m = floor(2^(31 + l) / d) + 1 (m < 2^32), floor(n m / 2^(31 + l))
+// is the quotient (Granlund and Montgomery 1994: m d - 2^(31 + l) <= d <= 2^l).
+struct Divider {
+    unsigned d, m, s;
+    explicit Divider(unsigned divisor) : d(divisor) {
+        int l = 0;
+        while ((1ull << l) < divisor) ++l;
+        m = (unsigned)((1ull << (31 + l)) / divisor + 1ull);
+        s = (unsigned)(l > 0 ? l - 1 : 0);
+        if (l == 0) m = 0u;                          // d = 1: n itself (div() below)
+    }
+    __device__ __forceinline__ unsigned div(unsigned n) const { return m ? __umulhi(n, m) >> s : n; }
+};
+
+// Field geometry for the boundary test of single cells.
+struct Geometry {
+    Divider nx, ny;
+    unsigned nz;
+    // Of the cells c + step j whose bit j is set in m (j < 4), those interior.
+    template <int STEP>
+    __device__ __forceinline__ unsigned interior(unsigned c, unsigned m) const {
+        unsigned row = nx.div(c), x = c - row * nx.d, z = ny.div(row), y = row - z * ny.d;
+        if (STEP == 1 && x + 3u < nx.d) {            // four cells of one row
+            const bool in = y - 1u < ny.d - 2u && z - 1u < nz - 2u;
+            if (x == 0u) m &= ~1u;
+            if (x + 4u == nx.d) m &= ~8u;
+            return in ? m : 0u;
+        }
+        unsigned k = 0u;
+        for (int j = 0; j < 4; ++j) {
+            const unsigned cj = c + (unsigned)(STEP * j);
+            row = nx.div(cj); x = cj - row * nx.d; z = ny.div(row); y = row - z * ny.d;
+            if (x - 1u < nx.d - 2u && y - 1u < ny.d - 2u && z - 1u < nz - 2u) k |= 1u << j;
+        }
+        return m & k;
+    }
+};
+
+// The values of a chunk: ALIGNED (16-byte aligned field): component k of v[u]
+// is cell c0 + 128 u + 4 lane + k; otherwise v[u] holds cells c0 + 128 u + 32 k
+// + lane.  Cells from `end` on read as 0.
+template <int U, bool ALIGNED>
+__device__ __forceinline__ void load_chunk(const float* __restrict__ phi, int64_t c0, int64_t end,
+                                           float4 (&v)[U]) {
     const int lane = threadIdx.x & 31;
-    unsigned w = m << (4 * (lane & 7));
-    w |= __shfl_xor_sync(0xffffffffu, w, 1);
-    w |= __shfl_xor_sync(0xffffffffu, w, 2);
-    w |= __shfl_xor_sync(0xffffffffu, w, 4);
-    if ((lane & 7) == 0 && x0 + 4 * lane < nx) fn((x0 >> 5) + (lane >> 3), w);
-}
-
-__device__ __forceinline__ float4 ld_row4(const float* __restrict__ row, bool ok, int x, int nx) {
-    return (ok && x < nx) ? __ldg(reinterpret_cast<const float4*>(row + x))
-                          : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-}
-
-// Pass 1.  Work is split by rows: warp w of a block takes rows w, w + 8, ...
-// of the block's tile.  A row's (y, z) is computed once per warp, rows on the
-// field boundary are skipped without reading them.  The per-tile count goes
-// to tile_count; with `bits` given, the row's interface bits are stored too
-// (wpr words per row), so that pass 3 need not read the field again.  In the
-// vector path a warp takes two rows at a time and issues the four 16-byte
-// loads per lane of 256 columns of both rows before using any of them, so
-// every lane keeps 64 bytes in flight (the pass is bound by load latency, not
-// by the compare work); rows of more than 512 cells are cut into 512-cell
-// segments, four loads per lane each (1024-cell rows: 0.26 -> 0.19 ms on a
-// 1 GiB field, the same as for 512-cell rows).  Eight blocks per SM (32
-// registers, a few bytes spilled) keep more loads in flight than the six that
-// 40 registers allow.
-__global__ void __launch_bounds__(CT_THREADS, 8)
-k_compact_count(const float* __restrict__ phi, int nx, int ny, int nz, int R, int64_t rows,
-                int* __restrict__ tile_count, unsigned* __restrict__ bits, int vec) {
-    pdl_wait();                                     // the kernel that wrote the field complete
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wpr = (nx + 31) >> 5;
-    const int64_t rbeg = (int64_t)blockIdx.x * R;
-    const int64_t rend = rbeg + R < rows ? rbeg + R : rows;
-    // rows < 2^31 (fields of at most 2^31 - 1 cells): 32-bit division
-    auto interior = [&](int64_t r) {
-        const unsigned z = (unsigned)r / (unsigned)ny, y = (unsigned)r - z * (unsigned)ny;
-        return y >= 1u && y + 2u <= (unsigned)ny && z >= 1u && z + 2u <= (unsigned)nz;
-    };
-    int cnt = 0;
-    if (vec && nx > 512) {
-        // long rows (fewer than 16 per tile): the tile's rows are cut into
-        // 512-cell segments (the last of a row partial), warp w takes segments
-        // w, w + 8, ..., and each lane issues its four 16-byte loads of a
-        // segment together, as in the two-row form below
-        const int spr = (nx + 511) >> 9;
-        const int nseg = (int)(rend - rbeg) * spr;
-        for (int sg = warp; sg < nseg; sg += CT_WARPS) {
-            const int rr = sg / spr;
-            const int x0 = (sg - rr * spr) << 9;
-            const int64_t r = rbeg + rr;
-            const bool ok = interior(r);
-            const float* row = phi + r * nx;
-            unsigned* br = bits ? bits + r * wpr : nullptr;
-            const int xa = x0 + 4 * lane;
-            float4 v[4];
+    if (c0 + 128 * U <= end) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = ld_row4(row, ok, xa + 128 * u, nx);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const unsigned m = ok ? nib4(v[u], xa + 128 * u, nx) : 0u;
-                cnt += __popc(m);
-                emit_nibbles(m, x0 + 128 * u, nx, [&](int w, unsigned b) { if (br) br[w] = b; });
+        for (int u = 0; u < U; ++u) {
+            if (ALIGNED) {
+                v[u] = __ldg(reinterpret_cast<const float4*>(phi + c0) + 32 * u + lane);
+            } else {
+                const float* p = phi + c0 + 128 * u + lane;
+                v[u] = make_float4(__ldg(p), __ldg(p + 32), __ldg(p + 64), __ldg(p + 96));
             }
         }
-        cnt = __reduce_add_sync(0xffffffffu, cnt);
-    } else if (vec) {
-        for (int64_t ra = rbeg + warp; ra < rend; ra += 2 * CT_WARPS) {
-            const int64_t rb = ra + CT_WARPS;
-            const bool oka = interior(ra), hasb = rb < rend, okb = hasb && interior(rb);
-            const float* rowa = phi + ra * nx;
-            const float* rowb = phi + (hasb ? rb : ra) * nx;
-            unsigned* ba = bits ? bits + ra * wpr : nullptr;
-            unsigned* bb = (bits && hasb) ? bits + rb * wpr : nullptr;
-            int ca = 0, cb = 0;
-            for (int x0 = 0; x0 < nx; x0 += 256) {
-                const int xa = x0 + 4 * lane, xb = xa + 128;
-                const float4 a0 = ld_row4(rowa, oka, xa, nx), a1 = ld_row4(rowa, oka, xb, nx);
-                const float4 b0 = ld_row4(rowb, okb, xa, nx), b1 = ld_row4(rowb, okb, xb, nx);
-                const unsigned ma0 = oka ? nib4(a0, xa, nx) : 0u, ma1 = oka ? nib4(a1, xb, nx) : 0u;
-                const unsigned mb0 = okb ? nib4(b0, xa, nx) : 0u, mb1 = okb ? nib4(b1, xb, nx) : 0u;
-                ca += __popc(ma0) + __popc(ma1);
-                cb += __popc(mb0) + __popc(mb1);
-                emit_nibbles(ma0, x0, nx, [&](int w, unsigned b) { if (ba) ba[w] = b; });
-                emit_nibbles(ma1, x0 + 128, nx, [&](int w, unsigned b) { if (ba) ba[w] = b; });
-                emit_nibbles(mb0, x0, nx, [&](int w, unsigned b) { if (bb) bb[w] = b; });
-                emit_nibbles(mb1, x0 + 128, nx, [&](int w, unsigned b) { if (bb) bb[w] = b; });
-            }
-            cnt += ca + cb;                       // the lane's share
-        }
-        cnt = __reduce_add_sync(0xffffffffu, cnt);
     } else {
-        for (int64_t r = rbeg + warp; r < rend; r += CT_WARPS) {
-            unsigned* rb = bits ? bits + r * wpr : nullptr;
-            if (!interior(r)) {
-                if (rb)
-                    for (int w = lane; w < wpr; w += 32) rb[w] = 0u;
-                continue;
-            }
-            const int c = row_bits(phi + r * nx, nx, false, [&](int w, unsigned b) {
-                if (rb) rb[w] = b;
-            });
-            cnt += c;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t c = c0 + 128 * u + (ALIGNED ? 4 * lane : lane);
+            constexpr int step = ALIGNED ? 1 : 32;
+            v[u].x = c < end ? __ldg(phi + c) : 0.0f;
+            v[u].y = c + step < end ? __ldg(phi + c + step) : 0.0f;
+            v[u].z = c + 2 * step < end ? __ldg(phi + c + 2 * step) : 0.0f;
+            v[u].w = c + 3 * step < end ? __ldg(phi + c + 3 * step) : 0.0f;
         }
     }
-    __shared__ int ws[CT_WARPS];
-    if (lane == 0) ws[warp] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int t = 0;
-#pragma unroll
-        for (int w = 0; w < CT_WARPS; ++w) t += ws[w];
-        tile_count[blockIdx.x] = t;
-    }
-    pdl_trigger();                                  // the next pass may be scheduled
 }
 
-// Pass 1 for 16-byte aligned rows of 128 * 2^k cells (the power-of-two edges
-// of the workloads), streamlined: the tile is a run of 128-cell slots (spr =
-// nx / 128 per row, 2^lspr), slot s of the tile is row s >> lspr at column
-// (s & (spr - 1)) * 128, so no column test is needed and a slot's bit words
-// are contiguous; warp w takes slots 4 w + u + 32 k and issues the four
-// 16-byte loads per lane of a trip together.  A row's (y, z) is stepped from
-// the tile's first row (a division only where the tile wraps to the next z).
-// The bits are the nibble layout of the general pass (word x / 32 of a row,
-// bit x % 32), so pass 3 is the same.
-__global__ void __launch_bounds__(CT_THREADS, 8)
-k_compact_count_p2(const float* __restrict__ phi, int nx, int ny, int nz, int R, int64_t rows,
-                   int lspr, int* __restrict__ tile_count, unsigned* __restrict__ bits) {
-    pdl_wait();                                     // the kernel that wrote the field complete
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t rbeg = (int64_t)blockIdx.x * R;
-    const int nr = (int)(rbeg + R < rows ? R : rows - rbeg);
-    const int nslot = nr << lspr;
-    const unsigned smask = (1u << lspr) - 1u;
-    const unsigned z0 = (unsigned)rbeg / (unsigned)ny, y0 = (unsigned)rbeg - z0 * (unsigned)ny;
-    const float4* base = reinterpret_cast<const float4*>(phi + rbeg * nx) + lane;
-    unsigned* tb = bits + (rbeg * nx >> 5) + (lane >> 3);
-    const unsigned shl = 4u * (unsigned)(lane & 7);
-    const bool writer = (lane & 7) == 0;
-    // the columns x = 0 and x = nx - 1 are lane 0's first and lane 31's last
-    // component of a row's first and last slot
-    const unsigned first_clear = lane == 0 ? 1u : 0u, last_clear = lane == 31 ? 8u : 0u;
-    int cnt = 0;
-    for (int s0 = warp * 4; s0 < nslot; s0 += 4 * CT_WARPS) {
-        float4 v[4];
-        bool ok[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int sl = s0 + u;
-            const unsigned row = (unsigned)sl >> lspr;
-            unsigned y = y0 + row, z = z0;
-            if (y >= (unsigned)ny) {                // the tile wraps to the next z plane
-                const unsigned k = y / (unsigned)ny;
-                z += k;
-                y -= k * (unsigned)ny;
-            }
-            ok[u] = sl < nslot && y - 1u < (unsigned)ny - 2u && z - 1u < (unsigned)nz - 2u;
-            v[u] = ok[u] ? __ldg(base + 32 * sl) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int sl = s0 + u;
-            const unsigned col = (unsigned)sl & smask;
-            unsigned m = (unsigned)iface_bits(__float_as_uint(v[u].x)) |
-                         ((unsigned)iface_bits(__float_as_uint(v[u].y)) << 1) |
-                         ((unsigned)iface_bits(__float_as_uint(v[u].z)) << 2) |
-                         ((unsigned)iface_bits(__float_as_uint(v[u].w)) << 3);
-            m &= ~((col == 0u ? first_clear : 0u) | (col == smask ? last_clear : 0u));
-            m = ok[u] ? m : 0u;
-            cnt += __popc(m);
-            unsigned w = m << shl;
-            w |= __shfl_xor_sync(0xffffffffu, w, 1);
-            w |= __shfl_xor_sync(0xffffffffu, w, 2);
-            w |= __shfl_xor_sync(0xffffffffu, w, 4);
-            if (writer && sl < nslot) tb[4 * sl] = w;
-        }
-    }
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
-    __shared__ int ws[CT_WARPS];
-    if (lane == 0) ws[warp] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int t = 0;
-#pragma unroll
-        for (int w = 0; w < CT_WARPS; ++w) t += ws[w];
-        tile_count[blockIdx.x] = t;
-    }
-    pdl_trigger();                                  // the next pass may be scheduled
+// The four-bit interface mask of a lane's component of a chunk, boundary
+// cells dropped: bit k for component k of v (see load_chunk), c its first cell.
+template <bool ALIGNED>
+__device__ __forceinline__ unsigned mask4(float4 v, unsigned c, const Geometry& g) {
+    unsigned m = (unsigned)iface_bits(v.x) | ((unsigned)iface_bits(v.y) << 1) |
+                 ((unsigned)iface_bits(v.z) << 2) | ((unsigned)iface_bits(v.w) << 3);
+    return m ? g.interior<ALIGNED ? 1 : 32>(c, m) : 0u;
 }
 
-// Pass 2: exclusive scan of ntiles ints by one block of 1024 threads, 32
-// consecutive entries per thread and round (eight 16-byte loads issued
-// together: one round up to 32 768 tiles, about 268 M cells); the total goes
-// to *d_count.  tile_count is 16-byte aligned (the workspace start).
-__global__ void __launch_bounds__(1024)
-k_compact_scan(int* __restrict__ tile_count, int64_t ntiles, int64_t* __restrict__ d_count) {
-    __shared__ long long wsum[32];
-    pdl_wait();                                     // pass 1 complete
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    long long carry = 0;
-    for (int64_t b0 = 0; b0 < ntiles; b0 += 32 * 1024) {
-        const int64_t i0 = b0 + 32 * (int64_t)threadIdx.x;
-        const bool full = i0 + 32 <= ntiles;
-        int v[32];
-        if (full) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int4 x = reinterpret_cast<const int4*>(tile_count + i0)[j];
-                v[4 * j] = x.x; v[4 * j + 1] = x.y; v[4 * j + 2] = x.z; v[4 * j + 3] = x.w;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = i0 + j < ntiles ? tile_count[i0 + j] : 0;
-        }
-        int own = 0;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) own += v[j];
-        long long x = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            long long w = wsum[lane];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const long long y = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += y;
-            }
-            wsum[lane] = w;
-        }
-        __syncthreads();
-        long long run = carry + (warp > 0 ? wsum[warp - 1] : 0) + x - own;
-        if (full) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                int4 o4;
-                o4.x = (int)run; run += v[4 * j];
-                o4.y = (int)run; run += v[4 * j + 1];
-                o4.z = (int)run; run += v[4 * j + 2];
-                o4.w = (int)run; run += v[4 * j + 3];
-                reinterpret_cast<int4*>(tile_count + i0)[j] = o4;
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                if (i0 + j < ntiles) tile_count[i0 + j] = (int)run;
-                run += v[j];
-            }
-        }
-        carry += wsum[31];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *d_count = carry;
-    pdl_trigger();
-}
-
-// Pass 3 without stored bits: each warp recomputes its rows' interface bits
-// from the field, the block scans the row counts, and every warp writes its
-// rows' indices at the row offsets, in ascending cell order.
+// Pass 1 (see the head of this file).  info[t]: the tile's count and, from bit
+// 16, its chunk mask (K * CT_WARPS bits; a count is at most 8192); super[b]:
+// the block's count (not written for S = 1).  Every chunk of a tile is loaded
+// before any is used (K U 16-byte loads per lane in flight).
+template <int U, int K, bool ALIGNED>
 __global__ void __launch_bounds__(CT_THREADS)
-k_compact_write(const float* __restrict__ phi, int nx, int ny, int nz, int R, int64_t rows,
-                const int* __restrict__ tile_offset, int32_t* __restrict__ idx, int64_t cap, int vec,
-                int64_t* __restrict__ d_count) {
-    __shared__ unsigned bal[CT_MAX_WORDS];
-    __shared__ int rowoff[CT_MAX_ROWS + 1];
-    __shared__ int rowcnt[CT_MAX_ROWS];
-    __shared__ long long s_base[CT_WARPS];
+k_compact_count(const float* __restrict__ phi, Geometry geo, int64_t base, int64_t cells, int64_t ntiles,
+                int S, int* __restrict__ info, int* __restrict__ super, unsigned* __restrict__ bits) {
+    constexpr int CHUNK = 128 * U, TILE = CT_WARPS * K * CHUNK;
+    __shared__ unsigned s_info[64];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    pdl_wait();                                     // the passes before complete
-    // with d_count given, tile_offset holds the per-tile counts of pass 1 and
-    // the block sums those of the tiles before its own (few tiles: no scan
-    // launch); the last block writes the total
-    if (d_count) {
-        long long part = 0;
-        for (int i = threadIdx.x; i < (int)blockIdx.x; i += CT_THREADS) part += __ldg(tile_offset + i);
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane == 0) s_base[warp] = part;
-    }
-    const int64_t rbeg = (int64_t)blockIdx.x * R;
-    const int64_t rend = rbeg + R < rows ? rbeg + R : rows;
-    const int nr = (int)(rend - rbeg);
-    const int wpr = (nx + 31) >> 5;                 // words per row
-    // the tile's bits are kept in shared memory when they fit, else each
-    // word is recomputed when it is written
-    const bool in_smem = (int64_t)nr * wpr <= CT_MAX_WORDS;
-    for (int k = warp; k < nr; k += CT_WARPS) {
-        const int64_t r = rbeg + k;
-        int cnt = 0;
-        const unsigned z = (unsigned)r / (unsigned)ny, y = (unsigned)r - z * (unsigned)ny;
-        if (y >= 1u && y + 2u <= (unsigned)ny && z >= 1u && z + 2u <= (unsigned)nz) {
-            cnt = row_bits(phi + r * nx, nx, vec != 0, [&](int w, unsigned b) {
-                if (in_smem) bal[k * wpr + w] = b;
-            });
-        } else if (in_smem) {
-            for (int w = lane; w < wpr; w += 32) bal[k * wpr + w] = 0u;
-        }
-        if (lane == 0) rowoff[k] = rowcnt[k] = cnt;
-    }
+    if (threadIdx.x < 64) s_info[threadIdx.x] = 0u;
     __syncthreads();
-    if (warp == 0) {
-        // exclusive scan of nr <= 1024 row counts: each lane sums a run of rows
-        const int per = (nr + 31) >> 5;
-        const int k0 = lane * per, k1 = min(k0 + per, nr);
-        int s = 0;
-        for (int k = k0; k < k1; ++k) s += rowoff[k];
-        int incl = s;
+    pdl_wait();                                     // the kernel that wrote the field complete
+    const int64_t t0 = (int64_t)blockIdx.x * S, end = base + cells;
+    const int nt = (int)(t0 + S < ntiles ? S : ntiles - t0);
+    for (int i = 0; i < nt; ++i) {
+        const int64_t first = base + (t0 + i) * TILE;
+        float4 v[K][U];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        int run = incl - s;
-        for (int k = k0; k < k1; ++k) {
-            const int c = rowoff[k];
-            rowoff[k] = run;
-            run += c;
-        }
-    }
-    __syncthreads();
-    int64_t base;
-    if (d_count) {
-        long long b = 0;
+        for (int q = 0; q < K; ++q) load_chunk<U, ALIGNED>(phi, first + (q * CT_WARPS + warp) * CHUNK, end, v[q]);
 #pragma unroll
-        for (int w = 0; w < CT_WARPS; ++w) b += s_base[w];
-        base = b;
-        if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *d_count = b + tile_offset[blockIdx.x];
-    } else {
-        base = tile_offset[blockIdx.x];
-    }
-    for (int k = warp; k < nr; k += CT_WARPS) {
-        if (rowcnt[k] == 0) continue;               // most rows of a field hold no interface cell
-        const int64_t r = rbeg + k;
-        int64_t pos = base + rowoff[k];
-        // one lane per 32-cell word: warp prefix of the word counts, then each
-        // lane writes its word's cells in order
-        for (int w0 = 0; w0 < wpr; w0 += 32) {
-            const int w = w0 + lane;
-            unsigned b = 0u;
-            if (w < wpr) {
-                if (in_smem) {
-                    b = bal[k * wpr + w];
+        for (int q = 0; q < K; ++q) {
+            float in[U], any = 0.0f;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                in[u] = max3(inside(v[q][u].x), inside(v[q][u].y), inside(v[q][u].z));
+                in[u] = fmaxf(in[u], inside(v[q][u].w));
+                any = fmaxf(any, in[u]);
+            }
+            if (!__any_sync(0xffffffffu, any > 0.0f)) continue;
+            const int64_t c0 = first + (q * CT_WARPS + warp) * CHUNK;
+            unsigned* wp = bits ? bits + ((c0 - base) >> 5) : nullptr;
+            int cnt = 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                unsigned m = 0u, w = 0u;
+                const bool some = __any_sync(0xffffffffu, in[u] > 0.0f);
+                if (some) m = mask4<ALIGNED>(v[q][u], (unsigned)(c0 + 128 * u + (ALIGNED ? 4 * lane : lane)), geo);
+                cnt += __popc(m);
+                if (!wp) continue;
+                if (ALIGNED) {
+                    if (some) {
+                        // the nibbles of 8 lanes make one word
+                        w = m << (4 * (lane & 7));
+                        w |= __shfl_xor_sync(0xffffffffu, w, 1);
+                        w |= __shfl_xor_sync(0xffffffffu, w, 2);
+                        w |= __shfl_xor_sync(0xffffffffu, w, 4);
+                    }
+                    if ((lane & 7) == 0) wp[4 * u + (lane >> 3)] = w;
                 } else {
-                    // recompute this word (rare: tiles of very long rows)
-                    const float* row = phi + r * nx;
-                    const unsigned z = (unsigned)r / (unsigned)ny, y = (unsigned)r - z * (unsigned)ny;
-                    if (y >= 1u && y + 2u <= (unsigned)ny && z >= 1u && z + 2u <= (unsigned)nz)
-                        for (int j = 0; j < 32; ++j) {
-                            const int x = 32 * w + j;
-                            if (x >= 1 && x <= nx - 2 && iface(__ldg(row + x))) b |= 1u << j;
-                        }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        w = __ballot_sync(0xffffffffu, (m >> k) & 1u);
+                        if (lane == 0) wp[4 * u + k] = w;
+                    }
                 }
             }
-            const int c = __popc(b);
+            cnt = __reduce_add_sync(0xffffffffu, cnt);
+            if (lane == 0 && cnt)
+                atomicAdd(&s_info[i], (unsigned)cnt | (0x10000u << (q * CT_WARPS + warp)));
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        int sum = 0;
+        for (int i = threadIdx.x; i < nt; i += 32) {
+            info[t0 + i] = (int)s_info[i];
+            sum += (int)(s_info[i] & 0xffffu);
+        }
+        if (S > 1) {
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            if (threadIdx.x == 0) super[blockIdx.x] = sum;
+        }
+    }
+    pdl_trigger();                                  // the next pass may be scheduled
+}
+
+// Pass 2: one warp per tile and trip, CT_WARPS * TPW consecutive tiles per
+// block (`tpw` trips; a block without cells returns at once).  The tile's first
+// slot is the sum of the counts before it: the block sums those of the blocks of
+// pass 1 before its first tile's (at most CT_MAX_SUPERS, eight 16-byte loads per
+// thread issued together), each warp adds those of the tiles from there to
+// its own.  With bits, the block lists the non-zero words of its eight tiles in
+// shared memory with their first slots (lane l of a tile's warp takes the words
+// W l .., W = TILE / 1024; words of unmarked chunks, never written, count as
+// 0; one warp scan), and then all its warps go through the list, lane q writing
+// bit q's cell: a short coalesced store per word, in parallel however the
+// cells crowd in one tile (a lane looping over the bits of its own words:
+// 836 k warp instructions on the 256^3 field; a warp going through its own
+// tile's words one after the other: 14 us).  Without bits the marked chunks are
+// read from the field again.  The warp of the last tile writes the total.
+template <int U, int K, bool ALIGNED, bool BITS>
+__global__ void __launch_bounds__(CT_THREADS)
+k_compact_emit(const float* __restrict__ phi, Geometry geo, int64_t base, int64_t cells, int64_t ntiles,
+               int S, int tpw, const int* __restrict__ info, const int* __restrict__ super,
+               const unsigned* __restrict__ bits, int32_t* __restrict__ idx, int64_t cap,
+               int64_t* __restrict__ d_count) {
+    constexpr int CHUNK = 128 * U, TILE = CT_WARPS * K * CHUNK, W = TILE / 1024;
+    __shared__ int s_part[CT_WARPS], s_words[CT_WARPS];
+    __shared__ uint2 s_list[BITS ? CT_WARPS * 32 * W : 1];
+    __shared__ unsigned short s_word[BITS ? CT_WARPS * 32 * W : 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nblk = CT_WARPS * tpw;                 // tiles of a block, at most 32
+    const int64_t t0 = (int64_t)blockIdx.x * nblk;
+    pdl_wait();                                     // pass 1 complete
+    // every warp holds the infos of the block's tiles, lane l tile t0 + l
+    const unsigned mine = (lane < nblk && t0 + lane < ntiles) ? (unsigned)__ldg(info + t0 + lane) : 0u;
+    const bool last = t0 + nblk >= ntiles;
+    if (!last && __all_sync(0xffffffffu, (mine & 0xffffu) == 0u)) return;
+    // the words of tile t0 + i of this warp (those of its marked chunks): lane l
+    // takes W of them, which lie in one chunk
+    static_assert((4 * U) % W == 0, "words and chunks nest");
+    unsigned b[W];
+    auto words = [&](int i) {
+        const unsigned marked = i < nblk ? __shfl_sync(0xffffffffu, mine, i) >> 16 : 0u;
+        const unsigned* tb = bits + (t0 + i) * (TILE / 32) + W * lane;
+        const bool on = (marked >> (W * lane / (4 * U))) & 1u;
+#pragma unroll
+        for (int k = 0; k < W; ++k) b[k] = on ? __ldg(tb + k) : 0u;
+    };
+    if constexpr (BITS) words(warp);                // one round trip with the sums below
+    // the block's first tile lies in pass-1 block b0 = t0 / S; the tiles from
+    // there to t0 are summed one by one (S and nblk are powers of two)
+    const int64_t b0 = t0 / S, r0 = b0 * S;
+    const int* head = S > 1 ? super : info;
+    const unsigned keep = S > 1 ? 0xffffffffu : 0xffffu;
+    unsigned part = 0u;                              // counts of fewer than 2^31 cells
+    {
+        const int n4 = (int)(b0 >> 2);
+        int4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int q = threadIdx.x + u * CT_THREADS;
+            v[u] = q < n4 ? __ldg(reinterpret_cast<const int4*>(head) + q) : make_int4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            part += (v[u].x & keep) + (v[u].y & keep) + (v[u].z & keep) + (v[u].w & keep);
+        if (threadIdx.x < (int)(b0 & 3)) part += __ldg(head + 4 * n4 + threadIdx.x) & keep;
+        if (threadIdx.x < (int)(t0 - r0)) part += __ldg(info + r0 + threadIdx.x) & 0xffff;
+    }
+    part = __reduce_add_sync(0xffffffffu, part);
+    if (lane == 0) s_part[warp] = (int)part;
+    __syncthreads();
+    unsigned before = 0u;
+#pragma unroll
+    for (int w = 0; w < CT_WARPS; ++w) before += (unsigned)s_part[w];
+    if (last && warp == 0) {
+        const unsigned total = before + __reduce_add_sync(0xffffffffu, mine & 0xffffu);
+        if (lane == 0) *d_count = (int64_t)total;
+    }
+    for (int i = warp; i < nblk; i += CT_WARPS) {
+        const unsigned own = __shfl_sync(0xffffffffu, mine, i);
+        int64_t pos = before + __reduce_add_sync(0xffffffffu, lane < i ? mine & 0xffffu : 0u);
+        const int64_t first = base + (t0 + i) * TILE;
+        if constexpr (BITS) {
+            // nothing in the eight tiles of this trip (the same for every warp)
+            if (!__any_sync(0xffffffffu, (lane & ~(CT_WARPS - 1)) == i - warp && mine != 0u)) {
+                words(i + CT_WARPS);
+                continue;
+            }
+            int c = 0;                               // cells, and non-zero words from bit 16
+#pragma unroll
+            for (int k = 0; k < W; ++k) c += __popc(b[k]) + (b[k] ? 0x10000 : 0);
             int incl = c;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
+                const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += u;
             }
-            int64_t p = pos + incl - c;
-            const int64_t cell0 = r * nx + 32 * (int64_t)w;
-            while (b) {
-                const int j = __ffs(b) - 1;
-                b &= b - 1u;
-                if (p < cap) idx[p] = (int32_t)(cell0 + j);
-                ++p;
+            if (lane == 31) s_words[warp] = incl >> 16;
+            __syncthreads();
+            int at = (incl - c) >> 16, total = 0;
+#pragma unroll
+            for (int w = 0; w < CT_WARPS; ++w) {
+                at += w < warp ? s_words[w] : 0;
+                total += s_words[w];
             }
-            pos += __shfl_sync(0xffffffffu, incl, 31);
-        }
-    }
-    pdl_trigger();
-}
-
-// Pass 3 with pass 1's interface bits: one warp per tile, a block of CT_WARPS
-// consecutive tiles.  The tile's base is the sum of the counts of the tiles
-// before it (fused: few tiles; the block sums the counts before its first
-// tile, each warp adds those of the block's tiles before its own, and the
-// warp of the last tile writes the total) or the exclusive offset written by
-// the scan launch (then the tile's count is the next offset, or the total,
-// minus its own).  A tile's words are contiguous (its rows, wpr words each):
-// each lane takes 8 consecutive words (two int4 loads when aligned), one warp
-// scan of the lane counts gives each lane its first slot, and the lane writes
-// its words' cells in ascending order.  One dependent load per tile (the
-// words, issued with the tile counts) and one barrier, in the fused prefix.
-__global__ void __launch_bounds__(CT_THREADS)
-k_compact_emit(int nx, int R, int64_t rows, int64_t ntiles, const int* __restrict__ tiles,
-               const unsigned* __restrict__ bits, int32_t* __restrict__ idx, int64_t cap,
-               int fused, int64_t* __restrict__ d_count) {
-    __shared__ long long s_part[CT_WARPS];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t t0 = (int64_t)blockIdx.x * CT_WARPS;
-    pdl_wait();                                     // the passes before complete
-    const int64_t t = t0 + warp;
-    const bool live = t < ntiles;
-    const int64_t rbeg = t * R;
-    const int nr = live ? (int)(rbeg + R < rows ? R : rows - rbeg) : 0;
-    const unsigned wpr = ((unsigned)nx + 31u) >> 5;
-    const int nw = nr * (int)wpr;
-    const unsigned* tb = bits + rbeg * (int64_t)wpr;
-    const bool al = ((rbeg * (int64_t)wpr) & 3) == 0;
-    // the lane's 8 words from word wl of the tile (none past the tile's end)
-    auto words = [&](unsigned (&b)[8], int wl) {
-        if (al && wl + 8 <= nw) {
-            const int4 x = __ldg(reinterpret_cast<const int4*>(tb + wl));
-            const int4 y = __ldg(reinterpret_cast<const int4*>(tb + wl + 4));
-            b[0] = x.x; b[1] = x.y; b[2] = x.z; b[3] = x.w;
-            b[4] = y.x; b[5] = y.y; b[6] = y.z; b[7] = y.w;
+            unsigned p = (unsigned)pos + (unsigned)((incl - c) & 0xffff);
+#pragma unroll
+            for (int k = 0; k < W; ++k)
+                if (b[k]) {
+                    s_list[at] = make_uint2(b[k], p);
+                    s_word[at] = (unsigned short)(32 * W * warp + W * lane + k);
+                    p += __popc(b[k]);
+                    ++at;
+                }
+            __syncthreads();
+            if (i + CT_WARPS < nblk) words(i + CT_WARPS);     // of the next trip
+            const unsigned cell0 = (unsigned)(base + (t0 + (i - warp)) * TILE) + lane;
+            const unsigned lt = (1u << lane) - 1u;
+#pragma unroll 4
+            for (int e = warp; e < total; e += CT_WARPS) {
+                const uint2 x = s_list[e];
+                const unsigned slot = x.y + __popc(x.x & lt);
+                if (((x.x >> lane) & 1u) && slot < cap) idx[slot] = (int32_t)(cell0 + 32u * s_word[e]);
+            }
+            __syncthreads();                         // the list is used again
         } else {
+            if ((own & 0xffffu) == 0u) continue;
+            for (unsigned todo = own >> 16; todo; todo &= todo - 1u) {
+                const int64_t c0 = first + (__ffs(todo) - 1) * CHUNK;
+                float4 v[U];
+                load_chunk<U, ALIGNED>(phi, c0, base + cells, v);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) b[k] = wl + k < nw ? __ldg(tb + wl + k) : 0u;
-        }
-    };
-    // the first 256 words of the tile are loaded before the tile counts are
-    // summed (the whole tile for rows of up to 256 cells): one round trip
-    unsigned b[8];
-    words(b, 8 * lane);
-    long long base = 0;
-    int tcount = 0;
-    if (fused) {
-        long long part = 0;
-        const int4* t4 = reinterpret_cast<const int4*>(tiles);
-        const int n4 = (int)(t0 >> 2);
-        int4 v[4];
+                for (int u = 0; u < U; ++u) {
+                    const int64_t c = c0 + 128 * u + (ALIGNED ? 4 * lane : lane);
+                    unsigned m = mask4<ALIGNED>(v[u], (unsigned)c, geo);
+                    if (ALIGNED) {
+                        int incl = __popc(m);
+                        const int n = incl;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int q = threadIdx.x + u * CT_THREADS;
-            v[u] = q < n4 ? __ldg(t4 + q) : make_int4(0, 0, 0, 0);
-        }
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+                            if (lane >= o) incl += x;
+                        }
+                        int64_t p = pos + incl - n;
+                        for (; m; m &= m - 1u, ++p)
+                            if (p < cap) idx[p] = (int32_t)(c + __ffs(m) - 1);
+                        pos += __shfl_sync(0xffffffffu, incl, 31);
+                    } else {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) part += (long long)v[u].x + v[u].y + v[u].z + v[u].w;
-        if (threadIdx.x < (int)(t0 & 3)) part += __ldg(tiles + 4 * n4 + threadIdx.x);
-        const int cj = (lane < CT_WARPS && t0 + lane < ntiles) ? __ldg(tiles + t0 + lane) : 0;
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane == 0) s_part[warp] = part;
-        __syncthreads();
-#pragma unroll
-        for (int w = 0; w < CT_WARPS; ++w) base += s_part[w];
-        base += __reduce_add_sync(0xffffffffu, lane < warp ? cj : 0);
-        tcount = __shfl_sync(0xffffffffu, cj, warp);
-        if (t == ntiles - 1 && lane == 0) *d_count = base + tcount;
-    } else {
-        if (!live) return;
-        base = __ldg(tiles + t);
-        const long long next = t + 1 < ntiles ? (long long)__ldg(tiles + t + 1) : *d_count;
-        tcount = (int)(next - base);
-    }
-    if (!live || tcount == 0) return;
-    const unsigned invw = wpr > 1u ? 0xFFFFFFFFu / wpr + 1u : 0u;
-    long long pos = base;
-    for (int w0 = 0; w0 < nw; w0 += 256) {
-        const int wl = w0 + 8 * lane;
-        if (w0 > 0) words(b, wl);
-        int c = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) c += __popc(b[k]);
-        int incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += u;
-        }
-        long long p = pos + incl - c;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            unsigned bb = b[k];
-            if (!bb) continue;
-            const unsigned w = (unsigned)(wl + k);
-            const unsigned r = wpr > 1u ? __umulhi(w, invw) : w, wr = w - r * wpr;
-            const int64_t cell0 = (rbeg + r) * (int64_t)nx + 32 * (int64_t)wr;
-            while (bb) {
-                const int q = __ffs(bb) - 1;
-                bb &= bb - 1u;
-                if (p < cap) idx[p] = (int32_t)(cell0 + q);
-                ++p;
+                        for (int k = 0; k < 4; ++k) {
+                            const unsigned w = __ballot_sync(0xffffffffu, (m >> k) & 1u);
+                            const int64_t p = pos + __popc(w & ((1u << lane) - 1u));
+                            if (((m >> k) & 1u) && p < cap) idx[p] = (int32_t)(c + 32 * k);
+                            pos += __popc(w);
+                        }
+                    }
+                }
             }
         }
-        pos += __shfl_sync(0xffffffffu, incl, 31);
     }
-    pdl_trigger();
+    pdl_trigger();                                  // (sooner: 1-4 us slower in all)
 }
 
-// The passes as programmatic dependent launches (launch_after): each waits
+// Both passes as programmatic dependent launches (launch_after): each waits
 // for the kernel before it on the stream, the first for the one that wrote
-// the field.
-static cudaError_t launch_count(const float* phi, int nx, int ny, int nz, int R, int64_t rows,
-                                int64_t nt, int* tiles, unsigned* bits, int vec, cudaStream_t s) {
-    void* args[] = {(void*)&phi, (void*)&nx, (void*)&ny, (void*)&nz, (void*)&R, (void*)&rows,
-                    (void*)&tiles, (void*)&bits, (void*)&vec};
-    return launch_after(reinterpret_cast<const void*>(&k_compact_count), dim3((unsigned)nt),
-                        dim3(CT_THREADS), args, s);
-}
-static cudaError_t launch_scan(int* tiles, int64_t nt, int64_t* d_count, cudaStream_t s) {
-    void* args[] = {(void*)&tiles, (void*)&nt, (void*)&d_count};
-    return launch_after(reinterpret_cast<const void*>(&k_compact_scan), dim3(1), dim3(1024), args, s);
-}
-static cudaError_t launch_write(const float* phi, int nx, int ny, int nz, int R, int64_t rows, int64_t nt,
-                                const int* tiles, int32_t* idx, int64_t cap, int vec, int64_t* d_count,
-                                cudaStream_t s) {
-    void* args[] = {(void*)&phi, (void*)&nx, (void*)&ny, (void*)&nz, (void*)&R, (void*)&rows,
-                    (void*)&tiles, (void*)&idx, (void*)&cap, (void*)&vec, (void*)&d_count};
-    return launch_after(reinterpret_cast<const void*>(&k_compact_write), dim3((unsigned)nt),
-                        dim3(CT_THREADS), args, s);
+// the field.  info: p.tiles ints, then (S > 1) p.supers ints from the next 16-byte
+// boundary; bits: one word per 32 of p.cells, whole tiles, or null.
+template <int U, int K, bool ALIGNED>
+static cudaError_t launch_compact(const float* phi, const Geometry& g, const CompactPlan& p, int* info,
+                                  unsigned* bits, int32_t* idx, int64_t cap, int64_t* d_count,
+                                  cudaStream_t s) {
+    Geometry geo = g;
+    int64_t base = p.base, cells = p.cells, tiles = p.tiles;
+    // two trips per block once the prefix is long (1 GiB: 224 us with the curvature
+    // after it, 226.5 with one trip, 225.4 with four)
+    int S = p.S, tpw = p.S > 1 ? 2 : 1;
+    int* super = info + (p.tiles + 3) / 4 * 4;
+    void* a1[] = {(void*)&phi, (void*)&geo, (void*)&base, (void*)&cells, (void*)&tiles,
+                  (void*)&S, (void*)&info, (void*)&super, (void*)&bits};
+    cudaError_t e = launch_after(reinterpret_cast<const void*>(&k_compact_count<U, K, ALIGNED>),
+                                 dim3((unsigned)p.supers), dim3(CT_THREADS), a1, s);
+    if (e != cudaSuccess) return e;
+    void* a2[] = {(void*)&phi, (void*)&geo, (void*)&base, (void*)&cells, (void*)&tiles, (void*)&S, (void*)&tpw,
+                  (void*)&info, (void*)&super, (void*)&bits, (void*)&idx, (void*)&cap, (void*)&d_count};
+    const void* k = bits ? reinterpret_cast<const void*>(&k_compact_emit<U, K, ALIGNED, true>)
+                         : reinterpret_cast<const void*>(&k_compact_emit<U, K, ALIGNED, false>);
+    return launch_after(k, dim3((unsigned)((p.tiles + CT_WARPS * tpw - 1) / (CT_WARPS * tpw))), dim3(CT_THREADS), a2, s);
 }
 
-// Tiles of a field: whole x-rows, tile_rows(nx) per tile.
-static int64_t compact_tiles(int nx, int64_t rows) {
-    const int R = tile_rows(nx);
-    return (rows + R - 1) / R;
+template <bool ALIGNED>
+static cudaError_t launch_compact(const float* phi, const Geometry& g, const CompactPlan& p, int* info,
+                                  unsigned* bits, int32_t* idx, int64_t cap, int64_t* d_count,
+                                  cudaStream_t s) {
+    if (p.tile == 8192) return launch_compact<4, 2, ALIGNED>(phi, g, p, info, bits, idx, cap, d_count, s);
+    if (p.tile == 4096) return launch_compact<4, 1, ALIGNED>(phi, g, p, info, bits, idx, cap, d_count, s);
+    return launch_compact<1, 1, ALIGNED>(phi, g, p, info, bits, idx, cap, d_count, s);
+}
+
+static cudaError_t compact_passes(const float* phi, int nx, int ny, int nz, const CompactPlan& p, int* info,
+                                  unsigned* bits, int32_t* idx, int64_t cap, int64_t* d_count,
+                                  cudaStream_t s) {
+    const Geometry g = {Divider((unsigned)nx), Divider((unsigned)ny), (unsigned)nz};
+    return aligned(phi, 16) ? launch_compact<true>(phi, g, p, info, bits, idx, cap, d_count, s)
+                            : launch_compact<false>(phi, g, p, info, bits, idx, cap, d_count, s);
+}
+
+// Ints of scratch before the bits: tile infos and block sums.
+static int64_t info_ints(const CompactPlan& p) {
+    return (p.tiles + 3) / 4 * 4 + (p.S > 1 ? p.supers : 0);
 }
 
 }  // namespace plic
@@ -631,11 +446,10 @@ extern "C" size_t plic_workspace_bytes(int op, int64_t arg) {
     if (arg < 0) return 0;
     switch (op) {
         case PLIC_WS_COMPACT: {
-            // tile counts: tiles hold >= CT_TILE/2 cells (or one whole row), so a
-            // field of arg cells has at most 2 arg / CT_TILE + 1 tiles; interface
-            // bits: one word per 32 cells of each row, at most arg / 16 words
-            // for rows of >= 32 cells (shorter rows keep no bits)
-            const int64_t t = (arg + plic::CT_TILE - 1) / plic::CT_TILE * 2 + 1;
+            // two words per 8192 cells and one per 16 cells: room for the tile
+            // infos and block sums (at most one word per 819 cells) and the
+            // interface bits (one word per 32 cells) of any field of arg cells
+            const int64_t t = (arg + 8191) / 8192 * 2 + 1;
             const size_t a = ((size_t)t * sizeof(int) + 255) / 256 * 256;
             const size_t b = ((size_t)(arg / 16 + 1) * sizeof(unsigned) + 255) / 256 * 256;
             return a + b;
@@ -667,65 +481,34 @@ extern "C" plic_status vof_interface_compact(const float* phi, int nx, int ny, i
     if (!phi || (!idx && idx_capacity > 0) || !workspace) return PLIC_ERR_ARG;
     if (ws_bytes < plic_workspace_bytes(PLIC_WS_COMPACT, ncell)) return PLIC_ERR_ARG;
     if (!aligned(phi, 4) || (idx && !aligned(idx, 4)) || !aligned(workspace, 256)) return PLIC_ERR_ALIGN;
-    const int64_t rows = (int64_t)ny * nz;
-    const int R = tile_rows(nx);
-    const int64_t nt = compact_tiles(nx, rows);
-    const size_t tile_bytes = ((size_t)nt * sizeof(int) + 255) / 256 * 256;
-    if (tile_bytes > ws_bytes) return PLIC_ERR_ARG;
-    int* tiles = reinterpret_cast<int*>(workspace);
-    const int64_t words = rows * ((nx + 31) / 32);
-    const size_t bits_bytes = ((size_t)words * sizeof(unsigned) + 255) / 256 * 256;
+    const CompactPlan p = compact_plan(nx, ny, nz);
+    int* info = reinterpret_cast<int*>(workspace);
+    const size_t info_bytes = ((size_t)info_ints(p) * sizeof(int) + 255) / 256 * 256;
+    // whole chunks of bits (512 cells)
+    const size_t bits_bytes = (size_t)((p.cells + 511) / 512) * 64;
     unsigned* bits = nullptr;
-    if (nx >= 32 && tile_bytes + bits_bytes <= ws_bytes)
-        bits = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(workspace) + tile_bytes);
-    const int vec = (nx % 4 == 0) && aligned(phi, 16);
-    // rows of 128 * 2^k cells: the streamlined count pass
-    int lspr = -1;
-    if (vec && bits && nx >= 128 && nx % 128 == 0 && ((nx / 128) & (nx / 128 - 1)) == 0)
-        for (lspr = 0; (128 << lspr) < nx; ++lspr) {}
-    cudaError_t e;
-    if (lspr >= 0) {
-        void* args[] = {(void*)&phi, (void*)&nx, (void*)&ny, (void*)&nz, (void*)&R, (void*)&rows,
-                        (void*)&lspr, (void*)&tiles, (void*)&bits};
-        e = launch_after(reinterpret_cast<const void*>(&k_compact_count_p2), dim3((unsigned)nt),
-                         dim3(CT_THREADS), args, s);
-    } else {
-        e = launch_count(phi, nx, ny, nz, R, rows, nt, tiles, bits, vec, s);
-    }
-    // up to CT_FUSED_SCAN_TILES tiles pass 3 sums the counts of the tiles
-    // before each block (at most that many L2 reads per block); beyond, one
-    // block scans them first
-    const bool fused = nt <= CT_FUSED_SCAN_TILES;
-    if (e == cudaSuccess && !fused) e = launch_scan(tiles, nt, d_count, s);
-    if (e == cudaSuccess) {
-        int fz = fused ? 1 : 0;
-        if (bits) {
-            const int64_t nb = (nt + CT_WARPS - 1) / CT_WARPS;
-            void* args[] = {(void*)&nx, (void*)&R, (void*)&rows, (void*)&nt, (void*)&tiles, (void*)&bits,
-                            (void*)&idx, (void*)&idx_capacity, (void*)&fz, (void*)&d_count};
-            e = launch_after(reinterpret_cast<const void*>(&k_compact_emit), dim3((unsigned)nb),
-                             dim3(CT_THREADS), args, s);
-        } else {
-            e = launch_write(phi, nx, ny, nz, R, rows, nt, tiles, idx, idx_capacity, vec,
-                             fused ? d_count : nullptr, s);
-        }
-    }
+    if (info_bytes + bits_bytes <= ws_bytes)
+        bits = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(workspace) + info_bytes);
+    else if (info_bytes > ws_bytes)
+        return PLIC_ERR_ARG;
+    const cudaError_t e = compact_passes(phi, nx, ny, nz, p, info, bits, idx, idx_capacity, d_count, s);
     if (e != cudaSuccess) { set_last_error("vof_interface_compact", e); return PLIC_ERR_CUDA; }
     return check_launch("vof_interface_compact");
 }
 
 // ---------------------------------------------------------------------------
-// Allocation-free variant.  The per-tile scratch of the three passes lives in
-// a file-scope device array instead of a caller-provided workspace.  Every
-// GPU that loads the library holds these 256 KiB until the process exits.
+// Allocation-free variant.  The scratch of the two passes (tile infos and block
+// sums, no bits) lives in a file-scope device array instead of a caller-provided
+// workspace.  Every GPU that loads the library holds these 256 KiB until the
+// process exits.
 // ---------------------------------------------------------------------------
 namespace plic {
 
-// one int per tile; a field of at most PLIC_NOALLOC_MAX_CELLS cells has at most
-// 2 * cells / CT_TILE + 1 tiles (see plic_workspace_bytes)
-constexpr int64_t kNoAllocMaxTiles = 2 * (PLIC_NOALLOC_MAX_CELLS / CT_TILE) + 1;
+// a field of at most PLIC_NOALLOC_MAX_CELLS cells has at most that many / 8192
+// tiles and CT_MAX_SUPERS block sums
+constexpr int64_t kNoAllocInts = 2 * (PLIC_NOALLOC_MAX_CELLS / 8192) + 1;
 
-static __device__ __align__(256) int g_noalloc_tiles[kNoAllocMaxTiles];
+static __device__ __align__(256) int g_noalloc_tiles[kNoAllocInts];
 
 // Device address of g_noalloc_tiles, looked up once per device (with that
 // device current) and cached; host code must not pass the symbol itself.
@@ -779,21 +562,12 @@ extern "C" plic_status vof_interface_compact_noalloc(const float* phi, int nx, i
     }
     // every tile entry that a pass reads is written earlier in the same call,
     // so the contents left by a previous call need no clearing
-    const int64_t rows = (int64_t)ny * nz;
-    const int R = tile_rows(nx);
-    const int64_t nt = compact_tiles(nx, rows);
-    if (nt > kNoAllocMaxTiles) {
+    const CompactPlan p = compact_plan(nx, ny, nz);
+    if (info_ints(p) > kNoAllocInts) {
         set_limit_error(ncell);
         return PLIC_ERR_ARG;
     }
-    // the built-in scratch holds the tile counts only; pass 3 re-reads the field
-    const int vec = (nx % 4 == 0) && aligned(phi, 16);
-    cudaError_t e = launch_count(phi, nx, ny, nz, R, rows, nt, tiles, nullptr, vec, s);
-    const bool fused = nt <= CT_FUSED_SCAN_TILES;
-    if (e == cudaSuccess && !fused) e = launch_scan(tiles, nt, d_count, s);
-    if (e == cudaSuccess)
-        e = launch_write(phi, nx, ny, nz, R, rows, nt, tiles, idx, idx_capacity, vec,
-                         fused ? d_count : nullptr, s);
+    const cudaError_t e = compact_passes(phi, nx, ny, nz, p, tiles, nullptr, idx, idx_capacity, d_count, s);
     if (e != cudaSuccess) { set_last_error("vof_interface_compact_noalloc", e); return PLIC_ERR_CUDA; }
     return check_launch("vof_interface_compact_noalloc");
 }
