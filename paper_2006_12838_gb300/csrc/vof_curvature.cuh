@@ -296,73 +296,90 @@ struct CellPlic {
     }
 };
 
+// Root of u^3 - 3 u + 2 a = 0 on 0 <= a <= 0.886, divided by 2/3: the
+// trigonometric root 2 sin(asin(a)/3) of cases (3)/(4) in units of t (Q = 3 t^2;
+// see p2::centre_distance).  The odd polynomial of p2::depressed_root (there with
+// powers of 3^(1/2) folded in), negated, then one Newton step, u <- (2/3) (a -
+// u^3)/(1 - u^2).
+struct UnitRoot {
+    static constexpr float c0 = -0.6675798892974854f, c1 = -0.07909464836120605f,
+                           c2 = -0.1595292091369629f, c3 = 0.23291343450546265f,
+                           c4 = -0.2261897623538971f;
+    static __device__ __forceinline__ float eval(float a) {
+        const float z = a * a;
+        const float n = a * fmaf(fmaf(fmaf(fmaf(c4, z, c3), z, c2), z, c1), z, c0);   // -u
+        const float v = n * n;
+        return fmaf(n, v, a) * rcp_approx(1.0f - v);
+    }
+};
+
 // The optimised SZ solution (Sec. 2.4) with everything that depends on the
 // normal alone computed once per curvature cell (all neighbour solves of a
 // cell use the centre normal, Eq. 36).  Per solve there remain: the reduced
 // volume, four threshold tests on V, the closed forms of cases (5), (2), (1)
-// (the last as cbrt(6 m1 m2 m3) * cbrt(V)), the trigonometric root of cases
-// (3)/(4) with the cancellation-free arcsine argument written as
-// (n1+n2 - 2 m3 V) s3 or (1 - 2V) s4, and the FP32 Newton polish of the
-// trigonometric root.  Same cases and formulas as solve_sz_opt_default; the
-// thresholds are the product-form tests divided through once.
+// (the last as cbrt(6 m1 m2 m3) * cbrt(V)), and the root of the depressed cubic
+// of cases (3)/(4) in units of t, whose argument a is linear in V: k3 V + a3 or
+// k4 V + a4 (p2::centre_distance; a clamped where the thresholds' rounding
+// lets a normal with m1 < 1e-14 m2 in).  All as distances s = 1/2 - d from the
+// cell's centre.  The thresholds are the product-form tests of
+// solve_sz_opt_default divided through once.
 template <>
 struct CellPlic<M_SZ_OPT> {
-    float L, m1, m2, m3, n12;
+    float L, m3;
     float V5, V1, V2, V3;
-    float s3, t3, s4, t4, k2a, k2b, cb1, inv1, k6;
+    float k3, a3, t3, b3, k4, a4, t4, k2a, k2b, h2, cb1;
     __device__ __forceinline__ void prepare(float nx, float ny, float nz) {
         const float ax = fabsf(nx), ay = fabsf(ny), az = fabsf(nz);
         L = ax + ay + az;
         // MUFU reciprocals (no IEEE division): the thresholds only choose
         // between case formulas that agree at the case boundaries
         const float il = rcp_approx(L);
-        m1 = fminf(fminf(ax, ay), az) * il;
+        const float m1 = fminf(fminf(ax, ay), az) * il;
         m3 = fmaxf(fmaxf(ax, ay), az) * il;
-        m2 = fmaxf(1.0f - (m1 + m3), 0.0f);
-        n12 = m1 + m2;
+        const float m2 = fmaxf(1.0f - (m1 + m3), 0.0f);
+        const float n12 = m1 + m2;
         const float m1m2 = m1 * m2, sq1 = m1 * m1;
         const float k23 = 6.0f * m2 * m3;
         const float rk = k23 > 0.0f ? rcp_approx(k23) : 0.0f;
-        inv1 = m1 > 0.0f ? rcp_approx(m1) : 0.0f;
+        const float inv1 = m1 > 0.0f ? rcp_approx(m1) : 0.0f;
         V5 = 0.5f * n12 * rcp_approx(m3);                  // case (5): V >= V5
         V1 = sq1 * rk;                                           // case (1): V < V1
         V2 = (sq1 - 3.0f * m2 * (m1 - m2)) * rk;                 // case (2): V < V2
         const float num3 = m3 * m3 * (3.0f * n12 - m3) + sq1 * (m1 - 3.0f * m3) + m2 * m2 * (m2 - 3.0f * m3);
         V3 = (m3 < n12 && m1m2 > 0.0f) ? num3 * rk * inv1 : 3.4e38f;  // case (3): V < V3
+        // case (3): t^2 = 2 m1 m2, a = 3/4 (m1 + m2 - 2 m3 V) / t
         const float t32 = 2.0f * m1m2;
-        const float r3 = t32 > 0.0f ? rsqrtf(t32) : 0.0f;
-        t3 = t32 * r3;
-        s3 = 1.5f * m1m2 * r3 * r3 * r3;
+        const float r3 = recip_sqrt(t32);
+        t3 = t32 * r3 * (2.0f / 3.0f);
+        a3 = 0.75f * n12 * r3;
+        k3 = -1.5f * m3 * r3;
+        b3 = 0.5f - n12;
+        // case (4): t^2 = (m1 (2 (m2 + m3) - m1) - (m3 - m2)^2)/4, a = 3/4 m1 m2 m3 (1 - 2 V) / t^3
         const float d32 = m3 - m2;
         const float t42 = 0.25f * (m1 * (2.0f * (m2 + m3) - m1) - d32 * d32);
-        const float r4 = t42 > 0.0f ? rsqrtf(t42) : 0.0f;
-        t4 = t42 * r4;
-        s4 = 0.75f * m1m2 * m3 * r4 * r4 * r4;
-        k2a = 8.0f * m2 * m3;
-        k2b = sq1 * (1.0f / 3.0f);
+        const float r4 = recip_sqrt(t42);
+        t4 = t42 * r4 * (2.0f / 3.0f);
+        a4 = 0.75f * m1m2 * m3 * r4 * r4 * r4;
+        k4 = -2.0f * a4;
+        k2a = 2.0f * m2 * m3;
+        k2b = sq1 * (1.0f / 12.0f);
+        h2 = 0.5f - 0.5f * m1;
         cb1 = Fm<float>::cbrt_(k23 * m1);
-        k6 = k23;
+    }
+    // 1/sqrt(x), 0 for x <= 0, with a Newton step (t and a carry its error)
+    static __device__ __forceinline__ float recip_sqrt(float x) {
+        const float r = x > 0.0f ? rsqrtf(x) : 0.0f;
+        return r * fmaf(-0.5f * x * r, r, 1.5f);
     }
     __device__ __forceinline__ float offset(float V0) const {
         const float V = fminf(V0, 1.0f - V0);
-        const bool c5 = V >= V5, c1 = V < V1, c2 = !c1 && V < V2, c3 = V < V3;
-        const float d5 = fmaf(m3, V, 0.5f * n12);
-        const float d2 = 0.5f * (m1 + Fm<float>::sqrt_(fmaxf(fmaf(k2a, V, -k2b), 1e-30f)));
-        const float d1 = cb1 * Fm<float>::cbrt_(V);
-        const float x = c3 ? fmaf(-2.0f * m3, V, n12) : fmaf(-2.0f, V, 1.0f);
-        const float arg = fminf(x * (c3 ? s3 : s4), 1.0f);
-        const float t = c3 ? t3 : t4, c = c3 ? n12 : 0.5f;
-        float d = fmaf(-2.0f * t, __sinf((1.0f / 3.0f) * fast_asinf(arg)), c);
-        // polish of the trigonometric root (cases 3/4: d >= m2, m1 > 0)
-        const float e2 = d - m2, e3 = fmaxf(d - m3, 0.0f);
-        const float e22 = e2 * e2, e33 = e3 * e3;
-        const float g = fmaf(3.0f * d, d - m1, m1 * m1) - fmaf(e22, e2, e33 * e3) * inv1 - k6 * V;
-        const float gp = fmaf(6.0f, d, -3.0f * m1) - 3.0f * (e22 + e33) * inv1;
-        d = d - g * rcp_approx(gp);
-        d = c1 ? d1 : d;
-        d = c2 ? d2 : d;
-        d = c5 ? d5 : d;
-        return L * copysignf(0.5f - d, V0 - 0.5f);
+        const bool c3 = V < V3;
+        float s = fmaf(c3 ? t3 : t4, UnitRoot::eval(fminf(fmaf(c3 ? k3 : k4, V, c3 ? a3 : a4), 0.9f)),
+                       c3 ? b3 : 0.0f);
+        if (V < V2) s = h2 - Fm<float>::sqrt_(fmaxf(fmaf(k2a, V, -k2b), 1e-30f));
+        if (V < V1) s = fmaf(-cb1, Fm<float>::cbrt_(V), 0.5f);
+        if (V >= V5) s = m3 * (0.5f - V);
+        return copysignf(L * s, V0 - 0.5f);
     }
 };
 
