@@ -55,6 +55,8 @@ def lib_path() -> str:
 def load():
     """Load libplic.so (built by ``paper_2006_12838_gb300.build.build()``)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -114,17 +116,40 @@ def _check(status: int, what: str):
                                        L.plic_last_error().decode()))
 
 
+# A call of a few thousand cells lasts as long as its Python: the helpers below
+# pass plain integers (ctypes converts them by the declared argument types) and
+# ask a tensor for nothing twice.  plic.offset on 4099 cells: 10.2 -> 5.4 us per call.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# the current stream's handle without a Stream object around it (2.0 us less)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(t, stream):
     if stream is not None:
-        return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
-    return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+        return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+    if _raw_stream is not None:
+        return _raw_stream(t.get_device())
+    return torch.cuda.current_stream(t.device).cuda_stream
 
 
 def _cuda(*ts, dtype=None):
+    ref = ts[0]
+    if ref.is_cuda:
+        dev = ref.get_device()
+        for t in ts:
+            if t is not None and (t.get_device() != dev or not t.is_contiguous()
+                                  or (dtype is not None and t.dtype is not dtype)):
+                break
+        else:
+            return
+    _refuse(ts, dtype)
+
+
+def _refuse(ts, dtype):
+    """Raise for the first argument that _cuda() found wrong."""
     ref = ts[0]
     for t in ts:
         if t is None:
@@ -254,9 +279,9 @@ def interface_compact(phi, idx=None, count=None, workspace=None, stream=None):
         idx = torch.empty(phi.numel(), dtype=torch.int32, device=phi.device)
     if count is None:
         count = torch.empty(1, dtype=torch.int64, device=phi.device)
-    ws_n = workspace_bytes(WS_COMPACT, phi.numel())
     if workspace is None:
-        workspace = torch.empty(max(ws_n, 1), dtype=torch.uint8, device=phi.device)
+        workspace = torch.empty(max(workspace_bytes(WS_COMPACT, phi.numel()), 1), dtype=torch.uint8,
+                                device=phi.device)
     _cuda(phi, idx, count, workspace)
     _check(load().vof_interface_compact(_ptr(phi), nx, ny, nz, _ptr(idx), idx.numel(), _ptr(count),
                                         _ptr(workspace), workspace.numel(),
@@ -320,9 +345,9 @@ def curvature_backward(phi, idx, g_kappa, n_iface=None, count=None, g_phi=None,
     n = idx.numel() if n_iface is None else int(n_iface)
     if g_phi is None:
         g_phi = torch.empty_like(phi)
-    ws_n = curv_bwd_workspace_bytes(phi.numel(), n)
     if workspace is None:
-        workspace = torch.empty(max(ws_n, 1), dtype=torch.uint8, device=phi.device)
+        workspace = torch.empty(max(curv_bwd_workspace_bytes(phi.numel(), n), 1), dtype=torch.uint8,
+                                device=phi.device)
     m = METHODS[method] if isinstance(method, str) else int(method)
     _check(load().vof_curvature_backward(_ptr(phi), nx, ny, nz, _ptr(idx), n, _ptr(count),
                                          _ptr(g_kappa), _ptr(g_phi), m, flags, _ptr(workspace),
