@@ -249,9 +249,11 @@ plic_status vof_laplace_pressure(const float *phi, int nx, int ny, int nz, const
  * curvature step of Sec. 4.2 and Appendix B: Eqs. 36, 38 and 42) with
  * respect to the fill field: g_phi = d(sum_k g_kappa[k] kappa[k]) / d phi,
  * with the interface set (idx and the neighbour flags 0 < phi < 1) held fixed.
- * g_phi is dense (nx*ny*nz floats) and overwritten.  Per interface cell the 27
+ * g_phi is dense (nx*ny*nz floats) and overwritten (during the call it also
+ * holds one mark per field cell).  Per interface cell the 27
  * partial derivatives are written to the workspace and gathered per field
- * cell, so the result is deterministic (no atomics).
+ * cell in a fixed order, so the result is deterministic (no floating-point
+ * atomics).
  * workspace: >= plic_curv_bwd_workspace_bytes(nx*ny*nz, n_iface) bytes,
  * 256-byte aligned; its contents on entry do not matter. */
 plic_status vof_curvature_backward(const float *phi, int nx, int ny, int nz,

@@ -22,46 +22,10 @@
 // The results equal those of the eight-lane layout up to the summation order
 // of the stencil sums and of the normal equations.
 #include "host_common.h"
-#include "plic_pair.cuh"
 #include "vof_curvature_coop.cuh"
+#include "vof_curvature_pair.cuh"
 
 namespace plic {
-
-// Offsets d0(V0, n) of two neighbours of a cell (both with the centre normal
-// of `pl`): for the optimised SZ solution, CellPlic<M_SZ_OPT>::offset on the
-// paired FP32 instructions (two neighbours per instruction; the case-(1) cube
-// root of the paired path); other methods solve one after the other.  These
-// solves are most of an interface cell's instructions, and the kernels are
-// issue bound: with the arcsine, the sine and a Newton step on Eq. 10 the batch of
-// 64 fields (2.59 M cells) took 252 us, with the root in units of t 207 us.
-template <int METHOD>
-__device__ __forceinline__ p2::f2 offset_two(const CellPlic<METHOD>& pl, p2::f2 V0) {
-    return make_float2(pl.offset(V0.x), pl.offset(V0.y));
-}
-template <>
-__device__ __forceinline__ p2::f2 offset_two<M_SZ_OPT>(const CellPlic<M_SZ_OPT>& P, p2::f2 V0) {
-    using namespace p2;
-    typedef UnitRoot R;
-    const f2 V = make_float2(fminf(V0.x, 1.0f - V0.x), fminf(V0.y, 1.0f - V0.y));
-    // the root of cases (3)/(4), as UnitRoot::eval
-    const b2 c3 = lt(V, mk(P.V3));
-    f2 a = fma(sel(c3, mk(P.k3), mk(P.k4)), V, sel(c3, mk(P.a3), mk(P.a4)));
-    a = make_float2(fminf(a.x, 0.9f), fminf(a.y, 0.9f));
-    const f2 z = mul(a, a);
-    f2 n = fma(mk(R::c4), z, mk(R::c3));
-    n = fma(n, z, mk(R::c2));
-    n = fma(n, z, mk(R::c1));
-    n = mul(a, fma(n, z, mk(R::c0)));
-    const f2 v = mul(n, n);
-    const f2 u = mul(fma(n, v, a), rcp(sub(mk(1.0f), v)));
-    f2 s = fma(sel(c3, mk(P.t3), mk(P.t4)), u, sel(c3, mk(P.b3), mk(0.0f)));
-    // cases (2), (1), (5)
-    s = sel(lt(V, mk(P.V2)), sub(mk(P.h2), sqrtp(fmax0(fma(mk(P.k2a), V, mk(-P.k2b))))), s);
-    s = sel(lt(V, mk(P.V1)), fma(mk(-P.cb1), cbrt_(V), mk(0.5f)), s);
-    s = sel(le(mk(P.V5), V), mul(mk(P.m3), sub(mk(0.5f), V)), s);
-    const f2 h = mul(mk(P.L), s);
-    return make_float2(copysignf(h.x, V0.x - 0.5f), copysignf(h.y, V0.y - 0.5f));
-}
 
 // kappa (sign per flags) of interface cell c of a field, one thread.
 template <int METHOD, int FIT>
