@@ -285,8 +285,9 @@ typedef struct {
  * concatenated logically, and
  * a grid of (#SMs x blocks_per_sm) blocks claims chunks of cells from a
  * device-side ticket counter until the work is exhausted (no waiting on other
- * blocks).  `fields` is a HOST array of n_fields descriptors; it is copied to
- * the workspace before the launch and may be reused once the call returns.
+ * blocks).  `fields` is a HOST array of n_fields descriptors; they go to the
+ * workspace by value (as kernel arguments, so a captured call keeps them) and
+ * the array may be reused once the call returns.
  * tuning: nullable (defaults are used).  workspace: >=
  * plic_workspace_bytes(PLIC_WS_BATCHED, n_fields) bytes, 256-byte aligned. */
 plic_status vof_curvature_batched(const vof_field *fields, int n_fields,

@@ -171,6 +171,7 @@ k_vof_curvature_batched_tpc(const vof_field* __restrict__ fields, const int64_t*
     const int lane = threadIdx.x & 31;
     __shared__ E27Shared tab;
     tab.fill();
+    pdl_wait();                  // the tables are written
     for (;;) {
         unsigned long long t = 0;
         if (lane == 0) t = atomicAdd(ticket, (unsigned long long)chunk);
