@@ -62,14 +62,19 @@ typedef enum {
 typedef enum {
     PLIC_FP32 = 0,           /* float in/out, fast-math solver                      */
     PLIC_FP32_POLISHED = 1,  /* float in/out, solver + one Newton step on Eq. 10    */
-    PLIC_FP64 = 2,           /* double in/out, the solver in double                 */
-    PLIC_FP64_REFINED = 3    /* double in/out, the FP32 solver (polished) on the
-                                reduced problem, then two Newton steps on Eq. 10
-                                in double-float arithmetic (48-bit significands on
-                                the FP32 pipes; doubles converted by integer bit
-                                operations, one FP64 add per cell): |d0 error| below
-                                1e-14 for |n| = 1, V0 >= 2^-126 (plic_offset only;
-                                the plane-sphere entries refine in FP64)        */
+    PLIC_FP64 = 2,           /* double in/out, the solver in double; plic_offset by
+                                the optimised SZ and the analytic solution (unless
+                                FAITHFUL) finishes an FP32 start by Newton steps in
+                                64-bit fixed point, rounded once: |d0 error| below
+                                6e-17 for |n| = 1                               */
+    PLIC_FP64_REFINED = 3    /* double in/out.  plic_offset by the optimised SZ and the
+                                analytic solution: as PLIC_FP64.  By the others: the
+                                FP32 solver (polished) on the reduced problem, then
+                                two Newton steps on Eq. 10 in double-float arithmetic
+                                (48-bit significands on the FP32 pipes; doubles
+                                converted by integer bit operations, one FP64 add per
+                                cell): |d0 error| below 1e-14 for |n| = 1, V0 >=
+                                2^-126.  The plane-sphere entries refine in FP64   */
 } plic_precision;
 
 enum {

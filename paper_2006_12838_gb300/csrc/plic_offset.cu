@@ -11,6 +11,7 @@
 // Roofline: 20 B/cell in FP32 (16 in, 4 out), 40 B/cell in FP64.  The FP32
 // solvers sit near the HBM/ALU balance point; FP64 is bound by the FP64 pipe.
 #include "host_common.h"
+#include "plic_fx.cuh"
 #include "plic_pair.cuh"
 #include "plic_solvers.cuh"
 
@@ -348,6 +349,61 @@ k_plic_offset_pair(const float* __restrict__ nx, const float* __restrict__ ny,
     if (COUNT) count_invalid(bad[0] + bad[1] + bad1[0], invalid);
 }
 
+// The optimised SZ and the analytic solution in PLIC_FP64 and
+// PLIC_FP64_REFINED: fx::offset, and the closed forms in FP64 for the cells it
+// refuses (a call, to keep their registers out of the loop).  Both methods and
+// precisions are this kernel: the offset is correctly rounded in nearly every cell,
+// and faster than the double-float steps of the other refined methods.
+// Bound: integer issue (641 warp instructions per 32 cells, every case of the
+// warp run through, 18.8 lanes on; ALU pipe 67 % busy).  2^24 cells: optimised
+// SZ 3200 us (closed forms, FP64 pipe 85 % busy) -> 379 us, analytic 4490 -> 380
+// us, 16 M cells FP64_REFINED 555 (double-float steps) -> 361 us; four blocks per
+// SM (64 registers) 379, at the compiler's 70 registers 401, five 383 us.
+template <int METHOD>
+__device__ __noinline__ double offset_cell_slow(double nx, double ny, double nz, double V0, int* bad) {
+    int b = 0;
+    const double r = offset_cell<METHOD, double, false, false>(nx, ny, nz, V0, b);
+    *bad += b;
+    return r;
+}
+
+template <int METHOD>
+__device__ __forceinline__ double offset_cell_fx(double nx, double ny, double nz, double V0, int& bad) {
+    typedef unsigned long long u64;
+    u64 d0;
+    if (fx::offset((u64)__double_as_longlong(nx), (u64)__double_as_longlong(ny), (u64)__double_as_longlong(nz),
+                   (u64)__double_as_longlong(V0), d0))
+        return __longlong_as_double((long long)d0);
+    return offset_cell_slow<METHOD>(nx, ny, nz, V0, &bad);
+}
+
+template <int METHOD, bool VEC>
+__global__ void __launch_bounds__(256, 4)
+k_plic_offset_fx(const double* __restrict__ nx, const double* __restrict__ ny,
+                 const double* __restrict__ nz, const double* __restrict__ V0, double* __restrict__ d0,
+                 int64_t n, int /* vec_ok: VEC */, unsigned long long* invalid, void* /* round trip: not fused here */) {
+    int bad = 0;
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t tail = 0;                                // the cells from here on go one at a time
+    if constexpr (VEC) {
+        const int64_t nvec = n / 2;
+        for (int64_t i = tid; i < nvec; i += stride) {
+            const double2 a = __ldcs(reinterpret_cast<const double2*>(nx) + i);
+            const double2 b = __ldcs(reinterpret_cast<const double2*>(ny) + i);
+            const double2 c = __ldcs(reinterpret_cast<const double2*>(nz) + i);
+            const double2 v = __ldcs(reinterpret_cast<const double2*>(V0) + i);
+            const double r0 = offset_cell_fx<METHOD>(a.x, b.x, c.x, v.x, bad);
+            const double r1 = offset_cell_fx<METHOD>(a.y, b.y, c.y, v.y, bad);
+            __stcs(reinterpret_cast<double2*>(d0) + i, make_double2(r0, r1));
+        }
+        tail = nvec * 2;
+    }
+    for (int64_t i = tail + tid; i < n; i += stride)
+        __stcs(d0 + i, offset_cell_fx<METHOD>(__ldcs(nx + i), __ldcs(ny + i), __ldcs(nz + i), __ldcs(V0 + i), bad));
+    count_invalid(bad, invalid);
+}
+
 // PLIC_FP64_REFINED: double in/out, FP32 solve + two FP64 Newton steps.
 template <int METHOD>
 __global__ void __launch_bounds__(256)
@@ -394,7 +450,15 @@ static const void* cptr() {
 // iterative solvers, packing wins (e.g. nested intervals FP32 27 -> 40, FP64
 // SZ-opt 3.3 -> 4.5 G solves/s).
 template <int METHOD>
-static const void* pick(plic_precision p, bool faithful) {
+static const void* pick(plic_precision p, bool faithful, bool vec) {
+    if constexpr (METHOD == M_SZ_OPT || METHOD == M_ANALYTIC) {
+        if (!faithful && (p == PLIC_FP64 || p == PLIC_FP64_REFINED))
+            return vec ? reinterpret_cast<const void*>(&k_plic_offset_fx<METHOD, true>)
+                       : reinterpret_cast<const void*>(&k_plic_offset_fx<METHOD, false>);
+        // in FP32 these two come here in their faithful forms only (pick_pair)
+        return p == PLIC_FP64 ? kptr<METHOD, double, false, true>()
+             : p == PLIC_FP32_POLISHED ? kptr<METHOD, float, true, true>() : kptr<METHOD, float, false, true>();
+    } else {
     if (p == PLIC_FP64_REFINED) return reinterpret_cast<const void*>(&k_plic_offset_refined<METHOD>);
     if (p == PLIC_FP64)
         return faithful ? kptr<METHOD, double, false, true>() : cptr<METHOD, double, false>();
@@ -404,6 +468,7 @@ static const void* pick(plic_precision p, bool faithful) {
                       : (faithful ? kptr<METHOD, float, true, true>() : kptr<METHOD, float, true, false>());
     return packed ? cptr<METHOD, float, false>()
                   : (faithful ? kptr<METHOD, float, false, true>() : kptr<METHOD, float, false, false>());
+    }
 }
 
 // The paired FP32 kernels (optimised SZ, Kawano's SZ, analytic); *fused is set
@@ -456,20 +521,20 @@ static plic_status offset_entry(const void* nx, const void* ny, const void* nz, 
         case PLIC_ANALYTIC:
             k = pair ? pick_pair<M_ANALYTIC>(p == PLIC_FP32_POLISHED, vrt != nullptr,
                                                             d_invalid_count != nullptr, vec_ok != 0, fused)
-                                    : pick<M_ANALYTIC>(p, faithful);
+                                    : pick<M_ANALYTIC>(p, faithful, vec_ok != 0);
             break;
         case PLIC_SZ_ORIG:
             k = pair ? pick_pair<M_SZ_ORIG>(p == PLIC_FP32_POLISHED, vrt != nullptr,
                                                            d_invalid_count != nullptr, vec_ok != 0, fused)
-                                    : pick<M_SZ_ORIG>(p, faithful);
+                                    : pick<M_SZ_ORIG>(p, faithful, vec_ok != 0);
             break;
         case PLIC_SZ_OPT:
             k = pair ? pick_pair<M_SZ_OPT>(p == PLIC_FP32_POLISHED, vrt != nullptr,
                                                           d_invalid_count != nullptr, vec_ok != 0, fused)
-                                    : pick<M_SZ_OPT>(p, faithful);
+                                    : pick<M_SZ_OPT>(p, faithful, vec_ok != 0);
             break;
-        case PLIC_NEWTON: k = pick<M_NEWTON>(p, faithful); break;
-        case PLIC_NESTED: k = pick<M_NESTED>(p, faithful); break;
+        case PLIC_NEWTON: k = pick<M_NEWTON>(p, faithful, vec_ok != 0); break;
+        case PLIC_NESTED: k = pick<M_NESTED>(p, faithful, vec_ok != 0); break;
     }
     const int threads = 256;
     const int W = dbl ? 2 : 4;
