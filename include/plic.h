@@ -65,8 +65,8 @@ typedef enum {
     PLIC_FP64 = 2,           /* double in/out, the solver in double; plic_offset by
                                 the optimised SZ and the analytic solution (unless
                                 FAITHFUL) finishes an FP32 start by Newton steps in
-                                64-bit fixed point, rounded once: |d0 error| below
-                                6e-17 for |n| = 1                               */
+                                64-bit fixed point: |d0 error| below 2e-16 for
+                                |n| = 1                                         */
     PLIC_FP64_REFINED = 3    /* double in/out.  plic_offset by the optimised SZ and the
                                 analytic solution: as PLIC_FP64.  By the others: the
                                 FP32 solver (polished) on the reduced problem, then

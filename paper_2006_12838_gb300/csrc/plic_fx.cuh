@@ -1,20 +1,21 @@
-// plic_fx.cuh -- the PLIC offset of a double cell to full double accuracy on
-// the integer and FP32 pipes (the optimised SZ and the analytic solution in
-// PLIC_FP64 and PLIC_FP64_REFINED).
+// plic_fx.cuh -- the PLIC offset of a double cell to full double accuracy, its
+// root on the integer and FP32 pipes (the optimised SZ and the analytic solution
+// in PLIC_FP64 and PLIC_FP64_REFINED).
 //
 // FP64 is scarce on GB300 (one FP64 operation per 72 FP32 ones), and the closed
-// forms take about 58 FP64 instructions per cell.  Here the reduced problem is
-// held in 64-bit fixed point (units of 2^-62), the cases are told apart from
-// linear combinations of it that are exact but for truncation, an FP32 start (18
-// bits) is formed for the unknown w of the case (p2::centre_distance: the depressed
-// cubic of cases (3)/(4), the cube of (1), the square of (2)), and two Newton
-// steps finish w: the residual once in fixed point, scaled by the exponents of the
-// normal so that its derivative is at least 3 units, the second step's by the
-// Taylor expansion of the polynomial about the start (exact: it is a cubic), with
-// the corrections in FP32.  The offset from the cell's centre, s = L/2 - d, is
-// summed in fixed point and rounded once: |d0 error| <= 5.9e-17 on 10^7 cells
-// against quadruple precision, where the closed forms reach 6e-16 (and the
-// double-float steps of the other refined methods 1.1e-14).
+// forms take about 58 FP64 instructions per cell.  Here six FP64 operations set the
+// reduced problem up (classify), an FP32 start (18 bits) is formed for the unknown w
+// of the case (p2::centre_distance: the depressed cubic of cases (3)/(4), the cube
+// of (1), the square of (2)), and two Newton steps finish w: the residual once
+// in 64-bit fixed point, scaled by the exponents of the normal so that its
+// derivative is at least 3 units, the second step's by the Taylor expansion of the
+// polynomial about the start (exact: it is a cubic), with the corrections in
+// FP32.  The offset from the cell's centre, s = L/2 - d, is summed in units of
+// 2^-62 and rounded once.  |d0 error| <= 1.8e-16 on 10^7 cells against quadruple
+// precision (rms 2.9e-17; the rounding of s, and of n1 + n2 and y in classify),
+// where the closed forms reach 8e-16 and the double-float steps of the other refined
+// methods 1.1e-14.  With the set-up in fixed point as well the error was 5.9e-17, but
+// the kernel 359 instead of 285 us.
 //
 // Cells outside the scheme's range (a normal far from unit length, 0 < V0 or
 // 1 - V0 below 2^-96, invalid input) and those whose steps do not come out as
@@ -38,6 +39,8 @@ FX_D u64 shl(u64 x, int s) { u64 r; asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(x)
 FX_D int clz(u64 x) { return __clzll((long long)x); }
 FX_D float asf(uint32_t u) { return __uint_as_float(u); }
 FX_D uint32_t asu(float f) { return __float_as_uint(f); }
+FX_D double asd(u64 u) { return __longlong_as_double((long long)u); }
+FX_D u64 bits(double d) { return (u64)__double_as_longlong(d); }
 FX_D float rsq(float x) { return rsqrtf(x); }
 FX_D float rcp(float x) { return rcp_approx(x); }
 FX_D float cbrt_start(float x) { return Fm<float>::exp2f_approx(Fm<float>::__log2f_approx(x) * (1.0f / 3.0f)); }
@@ -70,74 +73,62 @@ FX_D void sort(u64& b1, u64& b2, u64& b3) {
 }
 
 // Whether the scheme takes the cell (sorted |n|, V0's bits): n3 in [1/2, 1 +
-// 2^-20) and n1 < 3/4 (then L < 3), and V0 = 0 or in [2^-96, 1].
+// 2^-20) and n1 < 3/4 (then L < 3), and V0 = 0, in [2^-96, 1) or 1.
 FX_D bool in_range(u64 b1, u64 b3, u64 v0) {
-    const uint32_t h1 = (uint32_t)(b1 >> 32), h3 = (uint32_t)(b3 >> 32);
-    const u64 va = v0 & ABS;
-    return h3 - 0x3fe00000u <= 0x00100000u && h1 < 0x3fe80000u && va <= ONE &&
-           (va == 0ull || ((uint32_t)(va >> 32) >= (927u << 20) && (v0 >> 63) == 0ull));
+    const uint32_t h1 = (uint32_t)(b1 >> 32), h3 = (uint32_t)(b3 >> 32), hv = (uint32_t)(v0 >> 32);
+    return h3 - 0x3fe00000u <= 0x00100000u && h1 < 0x3fe80000u &&
+           (hv - (927u << 20) < 0x3ff00000u - (927u << 20) || (v0 & ABS) == 0ull || v0 == ONE);
 }
 
-constexpr float U62 = 2.168404344971009e-19f;        // 2^-62
-
-// A component's bits as n = M 2^(e - 64) with the leading bit of M set (M = 0
-// below 2^-61), and as a float (truncated to 24 bits).
-FX_D bool tiny(u64 b) { return (uint32_t)(b >> 32) < (962u << 20); }
-FX_D u64 mantissa(u64 b) { return tiny(b) ? 0ull : (b << 11) | TOP; }
+// A non-negative double's bits as M 2^(e - 64) with the leading bit of M set (M =
+// 0 below 2^-61), and in units of 2^-62 (truncated).
+FX_D u64 mantissa(u64 b) { return (uint32_t)(b >> 32) < (962u << 20) ? 0ull : (b << 11) | TOP; }
 FX_D int exponent(u64 b) { return (int)(b >> 52) - 1022; }
-FX_D float flt(u64 b) { return tiny(b) ? 0.0f : asf((uint32_t)(b >> 29) + 0x40000000u); }
+FX_D u64 fixed(u64 b) { return shr((b << 11) | TOP, 2 - exponent(b)); }
+// A double's magnitude as a float, truncated to 24 bits; 0 (a denormal) below 2^-127.  The
+// conversion instruction runs on the FP64 pipe: 572 us with it where these three
+// integer instructions take 396 (2^24 cells, at an earlier stage).
+FX_D float flt(u64 b) {
+    int t = (int)((uint32_t)(b >> 32) & 0x7fffffffu) - 0x38000000;
+    t = t > 0 ? t : 0;
+    return asf(((uint32_t)t << 3) | ((uint32_t)b >> 29));
+}
 
-// What the root of a case needs: n1 and n2 (bits), and in units of 2^-62
-//   (1), (2): n3 V = a 2^(ex - 64) (a normalised to 2 bits), s0 = L/2 or (n2 + n3)/2;
-//   (3): a = B = n1 + n2 - 2 n3 V, s0 = (n3 - n1 - n2)/2;
-//   (4): a = S5 = n3 (1/2 - V), s0 = n3.
+// What the root of a case needs, as doubles' bits: n1, n2, and
+//   (1): a = n3 V,             y = n1 + n2 + n3      (s = y/2 - w);
+//   (2): a = n3 V,             y = n2 + n3           (s = y/2 - w);
+//   (3): a = n1 + n2 - 2 n3 V, y = n3 - n1 - n2      (s = y/2 + w);
+//   (4): a = n3 (1/2 - V),     y = n3 - n1 - n2      (s = w).
 struct Task {
-    u64 b1, b2, a, s0;
-    int ex;
+    u64 b1, b2, a, y;
 };
 
-// The reduced problem of a cell (sorted |n|, |V0|): its case, 5 (then s is the
-// answer: n3 (1/2 - V), or L/2 for V = 0) or 1 to 4 (then t is filled).  Lengths
-// in units of 2^-62; V = min(V0, 1 - V0) = Mv 2^(ev - 64).
+// The case of a cell (sorted |n|, |V0|): 5, with s = n3 (1/2 - V) as a double's
+// bits, or 1 to 4, with t filled.  Six FP64 operations, the tests of
+// p2::centre_distance on floats.  B = n1 + n2 - 2 n3 V carries the rounding of n1 +
+// n2 (y too, with half the opposite effect on s); the tests stay sound however small
+// n1 is, since the cases meet to the third order and the test of cases (1)/(2) uses
+// the B of the root.
 FX_D int classify(u64 b1, u64 b2, u64 b3, u64 va, Task& t, u64& s) {
-    const u64 M3 = (b3 << 11) | TOP;
-    const int e3 = exponent(b3);
-    const u64 N1 = shr(mantissa(b1), 2 - exponent(b1)), N2 = shr(mantissa(b2), 2 - exponent(b2)),
-              N3 = shr(M3, 2 - e3);
-    const bool upper = va > HALF, zero = va == 0ull || va == ONE;
-    const u64 Mx = (va << 11) | TOP;
-    const int x = exponent(va);
-    u64 Vf = upper ? 0ull - Mx : shr(Mx, -x);        // V in units of 2^-64 (1 - V0 exactly)
-    if (zero) Vf = 0ull;
-    const u64 H = mulhi(N3, Vf), S5 = (N3 >> 1) - H, N12 = N1 + N2;
-    const i64 B = (i64)(N12 - (H << 1));
-    s = zero ? (N12 + N3) >> 1 : S5;
-    if (zero || B <= 0) return 5;
-    const int lz = clz(Vf | 1ull);
-    const u64 Mv = upper ? shl(Vf, lz) : Mx;
-    const int ev = upper ? -lz : x;
-    const float f1 = flt(b1), f2 = flt(b2), f3 = flt(b3);
-    const float fB = tof((u64)B) * U62, sq1 = f1 * f1;
+    const double n1 = asd(b1), n2 = asd(b2), n3 = asd(b3);
+    const double V = va > HALF ? 1.0 - asd(va) : asd(va);
+    const double h = n3 * V, n12 = n1 + n2;
+    const double B = fma(n3, asd(bits(V) + 0x8010000000000000ull), n12);         // - 2 V (V = 0: -2^-1022)
+    const double S5 = fma(-n3, V, asd(b3 - 0x0010000000000000ull));
+    s = bits(S5);
+    if ((i64)bits(B) <= 0) return 5;
+    const float f1 = flt(b1), f2 = flt(b2), fB = flt(bits(B)), sq1 = f1 * f1;
+    const bool c12 = 3.0f * f2 * fmaf(2.0f, f1, -fB) < sq1;
+    const bool c1 = c12 && 6.0f * f2 * flt(bits(h)) < sq1;
+    const double y = n3 + asd(c12 ? (c1 ? bits(n12) : b2) : bits(n12) ^ TOP);    // (selected before the one addition)
+    const float g = flt(bits(y));                    // n1 + n2 - n3, where y < 0
+    const bool c4 = !c12 && (i64)bits(y) < 0 && fmaf(g * g, g, 3.0f * f1 * f2 * fmaf(-2.0f, g, fB)) < 0.0f;
     t.b1 = b1;
     t.b2 = b2;
-    t.ex = e3 + ev;
-    if (3.0f * f2 * fmaf(2.0f, f1, -fB) < sq1) {
-        const float v48 = asf(((uint32_t)(Mv >> 40) & 0x7fffffu) | ((uint32_t)(ev + 174) << 23));  // V 2^48
-        const bool c1 = 6.0f * f2 * (f3 * v48) < sq1 * 2.81474976710656e14f;                       // 2^48
-        t.a = mulhi(M3, Mv);
-        t.s0 = (c1 ? N12 + N3 : N2 + N3) >> 1;
-        return c1 ? 1 : 2;
-    }
-    const i64 G = (i64)(N12 - N3);
-    const float g = G > 0 ? tof((u64)G) * U62 : 0.0f;
-    const bool c4 = G > 0 && fmaf(g * g, g, 3.0f * f1 * f2 * fmaf(-2.0f, g, fB)) < 0.0f;
-    t.a = c4 ? S5 : (u64)B;
-    t.s0 = c4 ? N3 : (u64)((i64)(N3 - N12) >> 1);
-    return c4 ? 4 : 3;
+    t.a = bits(c12 ? h : c4 ? S5 : B);
+    t.y = bits(y);
+    return c12 ? (c1 ? 1 : 2) : c4 ? 4 : 3;
 }
-
-// n3 V 2^48 of a task of case (1) or (2)
-FX_D float h48(const Task& t) { return (float)(uint32_t)(t.a >> 32) * exp2i(t.ex + 16); }
 
 // The two Newton steps from w = m 2^(j - 24): residual F, derivative P (units
 // of 2^-58, scaled alike), the polynomial's second and third Taylor coefficients
@@ -165,24 +156,25 @@ FX_D bool finish_root(uint32_t m, int j, i64 F, i64 P, float quad, float cubic, 
 
 // The start as m 2^(j - 24); false where w is below 2^-57 and counts as 0.
 FX_D bool split(float w, uint32_t& m, int& j) {
+    const bool some = w >= 6.938893903907228e-18f;
     w = w < 0.999f ? w : 0.999f;
     m = (asu(w) & 0x7fffffu) | 0x800000u;
     j = (int)(asu(w) >> 23) - 126;
-    return w >= 6.938893903907228e-18f;
+    return some;
 }
 
-// Case (2): w^2 = 2 n2 n3 V - n1^2/12, s = (n2 + n3)/2 - w.  The residual
-// 12 w^2 - 24 n2 n3 V + n1^2 scaled by 2^-j.
+// Case (2): w^2 = 2 n2 n3 V - n1^2/12.  The residual 12 w^2 - 24 n2 n3 V + n1^2
+// scaled by 2^-j.
 FX_D bool root_square(const Task& c, u64& s) {
     const float f1 = flt(c.b1);
-    const float t = fmaf(7.105427357601002e-15f * flt(c.b2), h48(c), f1 * f1 * -0.083333333333f);  // 2^-47
-    s = c.s0;
+    const float t = fmaf(2.0f * flt(c.b2), flt(c.a), f1 * f1 * -0.083333333333f);
+    s = fixed(c.y) >> 1;
     uint32_t m;
     int j;
-    if (!split(t * rsq(t), m, j)) return true;
+    if (!split(t * rsq(fmaxf(t, 1e-37f)), m, j)) return true;
     const u64 m2 = (u64)m * m, M1 = mantissa(c.b1);
     const u64 T = shr((m2 * 12ull) << 12, 4 - j) -
-                  shr(q3(mulhi(mantissa(c.b2), c.a)), j - (exponent(c.b2) + c.ex) + 3) +
+                  shr(q3(mulhi(mantissa(c.b2), ((c.a << 11) | TOP))), j - (exponent(c.b2) + exponent(c.a)) + 3) +
                   shr(mulhi(M1, M1), j - 2 * exponent(c.b1) + 8);
     u64 wt;
     const bool ok = finish_root(m, j, (i64)(T << 2), (i64)((u64)m * (24ull << 34)), 12.0f * exp2i(-j), 0.0f, wt);
@@ -190,23 +182,28 @@ FX_D bool root_square(const Task& c, u64& s) {
     return ok;
 }
 
-// Cases (3), (4): w^3 - Q w + R = 0 (p2::centre_distance), s = (n3 - n1 - n2)/2 +
-// w or w; case (1): w^3 = 6 n1 n2 n3 V, s = L/2 - w.  The residual 4 w^3 - 4 Q w
-// + 4 R scaled by 2^-(e1 + e2), or 4 w^3 - 24 n1 n2 n3 V by 2^-2j.
-FX_D bool root_cubic(const Task& c, int code, u64& s) {
-    const float f1 = flt(c.b1), f2 = flt(c.b2);
-    const bool c1 = code == 1, c4 = code == 4;
+// Cases (3), (4): w^3 - Q w + R = 0 (p2::centre_distance); case (1): w^3 =
+// 6 n1 n2 n3 V.  The residual 4 w^3 - 4 Q w + 4 R scaled by 2^-(e1 + e2), or
+// 4 w^3 - 24 n1 n2 n3 V by 2^-2j.
+template <int CODE>
+FX_D bool root_cubic(const Task& c, u64& s) {
+    const float f1 = flt(c.b1), f2 = flt(c.b2), fa = flt(c.a);
+    constexpr bool c1 = CODE == 1, c4 = CODE == 4;
+    const int e1 = exponent(c.b1), e2 = exponent(c.b2), ea = exponent(c.a);
+    const u64 M1 = mantissa(c.b1), M2 = mantissa(c.b2);
+    const i64 yh = (i64)(fixed(c.y & ABS) >> 1), Y = c.y >> 63 ? -yh : yh;       // y/2
+    const u64 N1 = shr(M1, 2 - e1), N2 = shr(M2, 2 - e2), N3 = N1 + N2 + (u64)(2 * Y);  // (case 4)
     float w;
     if (c1) {
-        w = cbrt_start(6.0f * f1 * (f2 * h48(c))) * 1.52587890625e-5f;           // 2^-16
+        w = cbrt_start(6.0f * f1 * (f2 * (fa * 2.81474976710656e14f))) * 1.52587890625e-5f;  // 2^48, 2^-16
     } else {
         const float p3 = 3.0f * f1 * f2;
         float Q = 2.0f * p3;
         if (c4) {
-            const float f3 = (float)(uint32_t)(c.s0 >> 32) * 9.31322574615478515625e-10f, d = f3 - f2;  // 2^-30
+            const float f3 = (float)(uint32_t)(N3 >> 32) * 9.31322574615478515625e-10f, d = f3 - f2;  // 2^-30
             Q = 0.75f * fmaf(f1, fmaf(2.0f, f2 + f3, -f1), -d * d);
         }
-        const float rq = rsq(Q), x = (p3 * rq) * (tof(c.a) * U62 * rq) * rq, z = x * x;
+        const float rq = rsq(Q), x = (p3 * rq) * (fa * rq) * rq, z = x * x;
         // 2 sin(asin(a)/3) as in p2::depressed_root, here to 5e-6 of itself
         float p = fmaf(483863.59375f, z, -151864.34375f);
         p = fmaf(p, z, 20440.373046875f);
@@ -217,21 +214,21 @@ FX_D bool root_cubic(const Task& c, int code, u64& s) {
         p = fmaf(p, z, 0.9999952912330627f);
         w = Q * rq * (x * p);
     }
-    s = c4 ? 0ull : c.s0;
+    s = c4 ? 0ull : (u64)Y;
     uint32_t m;
     int j;
     if (!split(w, m, j)) return true;
-    const int e1 = exponent(c.b1), e2 = exponent(c.b2), sc = c1 ? 2 * j : e1 + e2;
-    const u64 M1 = mantissa(c.b1), M2 = mantissa(c.b2);
-    const u64 m2 = (u64)m * m, P12 = mulhi(M1, M2), X = q3(mulhi(P12, c.a));
+    const int sc = c1 ? 2 * j : e1 + e2;
+    const u64 m2 = (u64)m * m, P12 = mulhi(M1, M2);
+    const u64 X = q3(mulhi(P12, c1 ? ((c.a << 11) | TOP) : fixed(c.a)));
     u64 q = c1 ? 0ull : P12 >> 1;
     if (c4) {
-        const u64 N1 = shr(M1, 2 - e1), N2 = shr(M2, 2 - e2), N3 = c.s0, D = N3 > N2 ? N3 - N2 : N2 - N3;
+        const u64 D = N3 > N2 ? N3 - N2 : N2 - N3;
         q = shr(mulhi(M1, ((N2 + N3) << 1) - N1), 2 + e2) - shl(mulhi(D, shl(D, -e1)), -e2);
     }
-    const u64 R = c1 ? 0ull - shr(X, 1 + 2 * j - (e1 + e2 + c.ex)) : X;
+    const u64 R = c1 ? 0ull - shr(X, 1 + 2 * j - (e1 + e2 + ea)) : X;
     const u64 w3 = (((m2 >> 24) * m) << 16) + (((m2 & 0xffffffull) * m) >> 8);
-    const i64 F = (i64)(shr(w3, 4 + sc - 3 * j) - shr(q3(mul24(q, m)), -j) + R);
+    const i64 F = (i64)(shr(w3, 4 + sc - 3 * j) - (c1 ? 0ull : shr(q3(mul24(q, m)), -j)) + R);
     const i64 P = (i64)(shr(q3(m2 << 16), 2 + sc - 2 * j) - q3(q));
     const float es = exp2i(-sc);
     u64 wt;
@@ -257,7 +254,12 @@ FX_D bool offset(u64 nx, u64 ny, u64 nz, u64 v0, u64& d0) {
     if (!in_range(b1, b3, v0)) return false;
     Task t;
     const int code = classify(b1, b2, b3, va, t, s);
-    const bool ok = code == 5 ? true : code == 2 ? root_square(t, s) : root_cubic(t, code, s);
+    if (code == 5) {
+        d0 = va < HALF ? s | TOP : s;
+        return true;
+    }
+    const bool ok = code == 2 ? root_square(t, s) : code == 3 ? root_cubic<3>(t, s)
+                  : code == 4 ? root_cubic<4>(t, s) : root_cubic<1>(t, s);
     d0 = round_s(s, va < HALF);
     return ok;
 }

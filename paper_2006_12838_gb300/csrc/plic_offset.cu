@@ -350,15 +350,8 @@ k_plic_offset_pair(const float* __restrict__ nx, const float* __restrict__ ny,
 }
 
 // The optimised SZ and the analytic solution in PLIC_FP64 and
-// PLIC_FP64_REFINED: fx::offset, and the closed forms in FP64 for the cells it
-// refuses (a call, to keep their registers out of the loop).  Both methods and
-// precisions are this kernel: the offset is correctly rounded in nearly every cell,
-// and faster than the double-float steps of the other refined methods.
-// Bound: integer issue (641 warp instructions per 32 cells, every case of the
-// warp run through, 18.8 lanes on; ALU pipe 67 % busy).  2^24 cells: optimised
-// SZ 3200 us (closed forms, FP64 pipe 85 % busy) -> 379 us, analytic 4490 -> 380
-// us, 16 M cells FP64_REFINED 555 (double-float steps) -> 361 us; four blocks per
-// SM (64 registers) 379, at the compiler's 70 registers 401, five 383 us.
+// PLIC_FP64_REFINED: the scheme of plic_fx.cuh, and the closed forms in FP64 for the
+// cells it refuses (a call, to keep their registers out of the loop).
 template <int METHOD>
 __device__ __noinline__ double offset_cell_slow(double nx, double ny, double nz, double V0, int* bad) {
     int b = 0;
@@ -367,40 +360,129 @@ __device__ __noinline__ double offset_cell_slow(double nx, double ny, double nz,
     return r;
 }
 
-template <int METHOD>
-__device__ __forceinline__ double offset_cell_fx(double nx, double ny, double nz, double V0, int& bad) {
-    typedef unsigned long long u64;
-    u64 d0;
-    if (fx::offset((u64)__double_as_longlong(nx), (u64)__double_as_longlong(ny), (u64)__double_as_longlong(nz),
-                   (u64)__double_as_longlong(V0), d0))
-        return __longlong_as_double((long long)d0);
-    return offset_cell_slow<METHOD>(nx, ny, nz, V0, &bad);
-}
+// Both methods and precisions are this kernel.  The cases are packed: FX_CELLS cells
+// per block and trip; every thread reads its four cells and settles case (5) and the
+// refused ones; the others leave their task in shared memory and their place in the
+// list of their case (lanes of one case share a counter's increment; the order in a
+// list does not matter); the warps take 32 cells of one list at a time; every thread
+// stores its own cells.  The arrays are read as integers: of the bits of a double in
+// a register the compiler makes |x| an operation on the FP64 pipe (three per cell:
+// 396 against 317 us).
+// Bound: integer issue (443 warp instructions per 32 cells, ALU pipe 60 % busy)
+// beside the FP64 pipe (7 instructions).  2^24 cells: closed forms 3200 us (optimised
+// SZ, FP64 pipe 85 % busy) and 4490 us (analytic); this scheme with one thread running
+// each of its cells through its case 379 us (every case of the warp in turn, 18.8 lanes
+// on) and with the tests in fixed point too; packed 285 us (28.4 lanes on).  16 M
+// cells FP64_REFINED 555 (double-float steps) -> 273 us.  256 threads and 1024 cells per
+// block 295 us, 64 and 256 295 us; ten blocks per SM (48 registers) 285, eight 287 us.
+// Below 2^15 cells 8.2 us at any shape (closed forms 18-22 us).
+constexpr int FX_THREADS = 128, FX_CELLS = 4 * FX_THREADS;
 
 template <int METHOD, bool VEC>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(FX_THREADS, 10)
 k_plic_offset_fx(const double* __restrict__ nx, const double* __restrict__ ny,
-                 const double* __restrict__ nz, const double* __restrict__ V0, double* __restrict__ d0,
-                 int64_t n, int /* vec_ok: VEC */, unsigned long long* invalid, void* /* round trip: not fused here */) {
+                        const double* __restrict__ nz, const double* __restrict__ V0,
+                        double* __restrict__ d0, int64_t n, int /* vec_ok: VEC */,
+                        unsigned long long* invalid, void* /* round trip: not fused here */) {
+    typedef fx::u64 u64;
+    typedef fx::i64 i64;
+    // a cell's task: b1 (with V0 < 1/2 in its sign), b2 and a, y; its d0 then in hi.y
+    __shared__ ulonglong2 lo[FX_CELLS], hi[FX_CELLS];
+    __shared__ unsigned short list[4][FX_CELLS];        // the cells of cases (1) to (4)
+    __shared__ int count[4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int bad = 0;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t tail = 0;                                // the cells from here on go one at a time
-    if constexpr (VEC) {
-        const int64_t nvec = n / 2;
-        for (int64_t i = tid; i < nvec; i += stride) {
-            const double2 a = __ldcs(reinterpret_cast<const double2*>(nx) + i);
-            const double2 b = __ldcs(reinterpret_cast<const double2*>(ny) + i);
-            const double2 c = __ldcs(reinterpret_cast<const double2*>(nz) + i);
-            const double2 v = __ldcs(reinterpret_cast<const double2*>(V0) + i);
-            const double r0 = offset_cell_fx<METHOD>(a.x, b.x, c.x, v.x, bad);
-            const double r1 = offset_cell_fx<METHOD>(a.y, b.y, c.y, v.y, bad);
-            __stcs(reinterpret_cast<double2*>(d0) + i, make_double2(r0, r1));
+    for (int64_t i0 = (int64_t)blockIdx.x * FX_CELLS; i0 < n; i0 += (int64_t)gridDim.x * FX_CELLS) {
+        const int cells = (int)(n - i0 < FX_CELLS ? n - i0 : FX_CELLS);
+        const bool vec = VEC && cells == FX_CELLS;
+        if (threadIdx.x < 4) count[threadIdx.x] = 0;
+        __syncthreads();
+        auto place = [&](int j) { return vec ? 2 * (FX_THREADS * (j >> 1) + (int)threadIdx.x) + (j & 1)
+                                             : FX_THREADS * j + (int)threadIdx.x; };
+        auto one = [&](int i, u64 ax, u64 ay, u64 az, u64 v) {
+            int code = 5;
+            if (i < cells) {
+                u64 b1 = ax & fx::ABS, b2 = ay & fx::ABS, b3 = az & fx::ABS;
+                const u64 va = v & fx::ABS, sign = va < fx::HALF ? fx::TOP : 0ull;
+                u64 s;
+                fx::sort(b1, b2, b3);
+                if (fx::in_range(b1, b3, v)) {
+                    fx::Task t;
+                    code = fx::classify(b1, b2, b3, va, t, s);
+                    if (code != 5) {
+                        lo[i] = make_ulonglong2(t.b1 | sign, t.b2);
+                        hi[i].x = t.a;
+                        s = t.y;
+                    } else {
+                        s |= sign;
+                    }
+                } else {
+                    s = fx::bits(offset_cell_slow<METHOD>(fx::asd(ax), fx::asd(ay), fx::asd(az), fx::asd(v), &bad));
+                }
+                hi[i].y = s;
+            }
+            const unsigned same = __match_any_sync(0xffffffffu, code);
+            const int first = __ffs(same) - 1;
+            int at = 0;
+            if (lane == first && code != 5) at = atomicAdd(&count[code - 1], __popc(same));
+            at = __shfl_sync(0xffffffffu, at, first) + __popc(same & ((1u << lane) - 1u));
+            if (code != 5) list[code - 1][at] = (unsigned short)i;
+        };
+        if (vec) {
+#pragma unroll 1
+            for (int k = 0; k < 2; ++k) {
+                const int64_t q = i0 / 2 + FX_THREADS * k + threadIdx.x;
+                const ulonglong2 a = __ldcs(reinterpret_cast<const ulonglong2*>(nx) + q);
+                const ulonglong2 b = __ldcs(reinterpret_cast<const ulonglong2*>(ny) + q);
+                const ulonglong2 c = __ldcs(reinterpret_cast<const ulonglong2*>(nz) + q);
+                const ulonglong2 d = __ldcs(reinterpret_cast<const ulonglong2*>(V0) + q);
+                one(place(2 * k), a.x, b.x, c.x, d.x);
+                one(place(2 * k + 1), a.y, b.y, c.y, d.y);
+            }
+        } else {
+#pragma unroll 1
+            for (int j = 0; j < 4; ++j) {
+                const int i = place(j);
+                const int64_t q = i0 + (i < cells ? i : 0);
+                one(i, __ldcs(reinterpret_cast<const u64*>(nx) + q), __ldcs(reinterpret_cast<const u64*>(ny) + q),
+                    __ldcs(reinterpret_cast<const u64*>(nz) + q), __ldcs(reinterpret_cast<const u64*>(V0) + q));
+            }
         }
-        tail = nvec * 2;
+        __syncthreads();
+        // 32 cells of a case at a time, the longest roots first
+        const int c1 = count[0], c2 = count[1], c3 = count[2], c4 = count[3];
+        const int t4 = (c4 + 31) >> 5, t3 = t4 + ((c3 + 31) >> 5), t1 = t3 + ((c1 + 31) >> 5),
+                  t2 = t1 + ((c2 + 31) >> 5);
+        for (int t = warp; t < t2; t += FX_THREADS / 32) {
+            const int code = t < t4 ? 4 : t < t3 ? 3 : t < t1 ? 1 : 2;
+            const int k = 32 * (t - (t < t4 ? 0 : t < t3 ? t4 : t < t1 ? t3 : t1)) + lane;
+            if (k < (code == 4 ? c4 : code == 3 ? c3 : code == 1 ? c1 : c2)) {
+                const int i = list[code - 1][k];
+                const ulonglong2 p = lo[i], q = hi[i];
+                const fx::Task c = {p.x & fx::ABS, p.y, q.x, q.y};
+                u64 s;
+                bool ok;
+                if (code == 2) ok = fx::root_square(c, s);
+                else if (code == 3) ok = fx::root_cubic<3>(c, s);
+                else if (code == 4) ok = fx::root_cubic<4>(c, s);
+                else ok = fx::root_cubic<1>(c, s);
+                hi[i].y = ok ? fx::round_s(s, (i64)p.x < 0)
+                             : fx::bits(offset_cell_slow<METHOD>(nx[i0 + i], ny[i0 + i], nz[i0 + i], V0[i0 + i], &bad));
+            }
+        }
+        __syncthreads();
+        if (vec) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                __stcs(reinterpret_cast<double2*>(d0) + i0 / 2 + FX_THREADS * k + threadIdx.x,
+                       make_double2(fx::asd(hi[place(2 * k)].y), fx::asd(hi[place(2 * k + 1)].y)));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (place(j) < cells) __stcs(d0 + i0 + place(j), fx::asd(hi[place(j)].y));
+        }
+        // (the next trip writes the tasks behind its first barrier)
     }
-    for (int64_t i = tail + tid; i < n; i += stride)
-        __stcs(d0 + i, offset_cell_fx<METHOD>(__ldcs(nx + i), __ldcs(ny + i), __ldcs(nz + i), __ldcs(V0 + i), bad));
     count_invalid(bad, invalid);
 }
 
@@ -462,11 +544,11 @@ static const void* pick(plic_precision p, bool faithful, bool vec) {
     if (p == PLIC_FP64_REFINED) return reinterpret_cast<const void*>(&k_plic_offset_refined<METHOD>);
     if (p == PLIC_FP64)
         return faithful ? kptr<METHOD, double, false, true>() : cptr<METHOD, double, false>();
-    const bool packed = !faithful && METHOD != M_SZ_ORIG;
+    const bool compact = !faithful && METHOD != M_SZ_ORIG;
     if (p == PLIC_FP32_POLISHED)
-        return packed ? cptr<METHOD, float, true>()
+        return compact ? cptr<METHOD, float, true>()
                       : (faithful ? kptr<METHOD, float, true, true>() : kptr<METHOD, float, true, false>());
-    return packed ? cptr<METHOD, float, false>()
+    return compact ? cptr<METHOD, float, false>()
                   : (faithful ? kptr<METHOD, float, false, true>() : kptr<METHOD, float, false, false>());
     }
 }
@@ -516,6 +598,7 @@ static plic_status offset_entry(const void* nx, const void* ny, const void* nz, 
                        aligned(d0, 16) && (!vrt || aligned(vrt, 16));
     const bool faithful = (flags & PLIC_FLAG_FAITHFUL) != 0;
     const bool pair = !dbl && !faithful && (m == PLIC_ANALYTIC || m == PLIC_SZ_ORIG || m == PLIC_SZ_OPT);
+    const bool fx = dbl && !faithful && (m == PLIC_ANALYTIC || m == PLIC_SZ_OPT);
     const void* k = nullptr;
     switch (m) {
         case PLIC_ANALYTIC:
@@ -536,10 +619,11 @@ static plic_status offset_entry(const void* nx, const void* ny, const void* nz, 
         case PLIC_NEWTON: k = pick<M_NEWTON>(p, faithful, vec_ok != 0); break;
         case PLIC_NESTED: k = pick<M_NESTED>(p, faithful, vec_ok != 0); break;
     }
-    const int threads = 256;
-    const int W = dbl ? 2 : 4;
-    // 4 cells per thread also where the paired kernels read unaligned arrays
-    const int64_t work = vec_ok || pair ? (n + W - 1) / W : n;
+    const int threads = fx ? FX_THREADS : 256;
+    const int W = dbl && !fx ? 2 : 4;
+    // 4 cells per thread also where the paired and the packed FP64 kernels read
+    // unaligned arrays
+    const int64_t work = vec_ok || pair || fx ? (n + W - 1) / W : n;
     const int grid = stream_grid(k, threads, work);
     unsigned long long* inv = reinterpret_cast<unsigned long long*>(d_invalid_count);
     void* args[] = {(void*)&nx, (void*)&ny, (void*)&nz, (void*)&V0, (void*)&d0,

@@ -28,6 +28,8 @@ FX_D u64 shr(u64 x, int s) { bad_shifts += s < 0 && x; return s < 0 || s > 63 ? 
 FX_D u64 shl(u64 x, int s) { bad_shifts += s < 0 && x; return s < 0 || s > 63 ? 0 : x << s; }
 FX_D int clz(u64 x) { return x ? __builtin_clzll(x) : 64; }
 FX_D float asf(uint32_t u) { float f; memcpy(&f, &u, 4); return f; }
+FX_D double asd(u64 u) { double d; memcpy(&d, &u, 8); return d; }
+FX_D u64 bits(double d) { u64 u; memcpy(&u, &d, 8); return u; }
 FX_D uint32_t asu(float f) { uint32_t u; memcpy(&u, &f, 4); return u; }
 FX_D float rsq(float x) { return (float)(1 / std::sqrt((double)x) * off(1.2e-7)); }
 FX_D float rcp(float x) { return (float)(1 / (double)x * off(1.2e-7)); }

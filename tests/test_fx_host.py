@@ -1,8 +1,9 @@
 """The fixed-point FP64 offset on the host (the same source as on the GPU),
-against quadruple precision: |d0 error| <= 6e-17, half an ulp of numbers up to
-0.87 (5.55e-17) and the root's own error (a few units of 2^-58 over a derivative
-of at least 3); no cell inside the scheme's range is refused, no shift count is
-negative."""
+against quadruple precision: |d0 error| <= 2e-16, the sum of half an ulp of numbers
+up to 0.87 (5.6e-17), of y/2 with y up to 1.74 (5.6e-17) and of half the rounding of
+n1 + n2 up to 1.41 (5.6e-17), and the root's own error (a few units of 2^-58 over a
+derivative of at least 3); no cell inside the scheme's range is refused, no shift
+count is negative."""
 import os
 import shutil
 import subprocess
@@ -25,4 +26,4 @@ def exe(tmp_path_factory):
 def test_against_quadruple_precision(exe, kind):
     r = subprocess.run([exe, "40000", str(kind)], check=True, capture_output=True, text=True)
     refused, worst, shifts = r.stdout.split()
-    assert (int(refused), int(shifts)) == (0, 0) and float(worst) <= 6e-17, r.stdout
+    assert (int(refused), int(shifts)) == (0, 0) and float(worst) <= 2e-16, r.stdout

@@ -10,8 +10,8 @@ import torch
 from paper_2006_12838_gb300 import plic
 
 pytestmark = pytest.mark.gpu
-# d0 <= 0.87 is rounded once (5.6e-17) after a root within 2e-18; the oracle's own bisection
-# on doubles is within 4e-16 of the offset (a few ulp of L/2 and of the volume over an
+# d0 is within 2e-16 (tests/test_fx_host.py); the oracle's own bisection
+# on doubles is within 3e-16 of the offset (a few ulp of L/2 and of the volume over an
 # area of at least 0.1); volumes below are in [1e-3, 1 - 1e-3] for this bound
 TIGHT = 5e-16
 # the FP64 bound for all volumes: where the cut polygon degenerates the oracle's
