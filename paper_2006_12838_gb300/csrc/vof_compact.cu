@@ -47,10 +47,12 @@ struct CompactPlan {
     int tile, S;
 };
 
-// Tile sizes: 8192 cells (16 loads of 16 bytes per lane in flight) where the
-// field gives every SM several blocks of it, smaller tiles below, where the
-// pass lasts as long as one block (64^3: 248 tiles of 1024 cells 5.9 us, 32 tiles
-// of 8192 14 us).  S grows once the write pass would have to sum more
+// Tile sizes: 8192 cells (16 loads of 16 bytes per lane in flight) where that
+// fills the chip more than twice (2560 blocks and up), smaller tiles below, where
+// the last blocks and, smaller still, a single block set the time (64^3: 248 tiles
+// of 1024 cells 5.9 us, 32 tiles of 8192 14 us; with the curvature after it, 256^3
+// 24.0 us with 8192 cells and 23.6 with 4096, 301 x 203 x 257 24.0 and 23.7,
+// 1 GiB 215 and 219).  S grows once the write pass would have to sum more
 // than CT_MAX_SUPERS counts (above 67 M cells; one scan launch in between took
 // 11 us on 1 GiB).
 static CompactPlan compact_plan(int nx, int ny, int nz) {
@@ -58,7 +60,7 @@ static CompactPlan compact_plan(int nx, int ny, int nz) {
     const int64_t nxy = (int64_t)nx * ny;
     p.base = nxy & ~(int64_t)31;
     p.cells = nxy * (nz - 1) - p.base;
-    p.tile = p.cells >= (int64_t)5 << 20 ? 8192 : p.cells >= (int64_t)1 << 20 ? 4096 : 1024;
+    p.tile = p.cells >= (int64_t)20 << 20 ? 8192 : p.cells >= (int64_t)1 << 20 ? 4096 : 1024;
     p.tiles = (p.cells + p.tile - 1) / p.tile;
     p.S = 1;
     while ((p.tiles + p.S - 1) / p.S > CT_MAX_SUPERS) p.S *= 2;
