@@ -8,6 +8,7 @@
 // a grid-stride loop on up to 16 waves of blocks (stream_grid), as plic_offset
 // does.
 #include "host_common.h"
+#include "plic_adjoint64.cuh"
 #include "plic_polygon.cuh"
 
 namespace plic {
@@ -94,6 +95,61 @@ k_plic_adjoint(const T* __restrict__ nx, const T* __restrict__ ny, const T* __re
     }
 }
 
+// The FP64 adjoints: area_centroid64 on the values' bits, the cells it refuses by
+// adjoint_cell (a call, to keep its registers out of the loop).  Bound: the FP64
+// pipe (62 operations per cell); 16-byte vectors as above.
+template <int MODE>
+__device__ __noinline__ void adjoint_cell_slow(fx::u64 nx, fx::u64 ny, fx::u64 nz, fx::u64 d0, double g, double* o) {
+    adjoint_cell<double, MODE>(fx::asd(nx), fx::asd(ny), fx::asd(nz), fx::asd(d0), g, o[0], o[1], o[2], o[3]);
+}
+
+template <int MODE>
+__device__ __forceinline__ void adjoint_cell64(fx::u64 nx, fx::u64 ny, fx::u64 nz, fx::u64 d0, double g, double& gs,
+                                               double& gx, double& gy, double& gz) {
+    double A, cx, cy, cz;                            // MODE 0: 1/A
+    if (fx::area_centroid64<MODE == 0>(nx, ny, nz, d0, A, cx, cy, cz)) {
+        gs = g * A;
+        const double s = MODE == 0 ? g : -gs;
+        gx = s * cx; gy = s * cy; gz = s * cz;
+    } else {
+        double o[4];
+        adjoint_cell_slow<MODE>(nx, ny, nz, d0, g, o);
+        gs = o[0]; gx = o[1]; gy = o[2]; gz = o[3];
+    }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(256)
+k_plic_adjoint64(const fx::u64* __restrict__ nx, const fx::u64* __restrict__ ny, const fx::u64* __restrict__ nz,
+                 const fx::u64* __restrict__ d0, const double* __restrict__ g, double* __restrict__ gs,
+                 double* __restrict__ gx, double* __restrict__ gy, double* __restrict__ gz, int64_t n, int vec_ok) {
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t nvec = vec_ok ? n / 2 : 0;
+    for (int64_t i = tid; i < nvec; i += stride) {
+        const ulonglong2 a = __ldcs(reinterpret_cast<const ulonglong2*>(nx) + i);
+        const ulonglong2 b = __ldcs(reinterpret_cast<const ulonglong2*>(ny) + i);
+        const ulonglong2 c = __ldcs(reinterpret_cast<const ulonglong2*>(nz) + i);
+        const ulonglong2 d = __ldcs(reinterpret_cast<const ulonglong2*>(d0) + i);
+        const double2 e = __ldcs(reinterpret_cast<const double2*>(g) + i);
+        double2 o0, o1, o2, o3;
+        adjoint_cell64<MODE>(a.x, b.x, c.x, d.x, e.x, o0.x, o1.x, o2.x, o3.x);
+        adjoint_cell64<MODE>(a.y, b.y, c.y, d.y, e.y, o0.y, o1.y, o2.y, o3.y);
+        if (gs) __stcs(reinterpret_cast<double2*>(gs) + i, o0);
+        if (gx) __stcs(reinterpret_cast<double2*>(gx) + i, o1);
+        if (gy) __stcs(reinterpret_cast<double2*>(gy) + i, o2);
+        if (gz) __stcs(reinterpret_cast<double2*>(gz) + i, o3);
+    }
+    for (int64_t i = nvec * 2 + tid; i < n; i += stride) {
+        double o0, o1, o2, o3;
+        adjoint_cell64<MODE>(nx[i], ny[i], nz[i], d0[i], g[i], o0, o1, o2, o3);
+        if (gs) gs[i] = o0;
+        if (gx) gx[i] = o1;
+        if (gy) gy[i] = o2;
+        if (gz) gz[i] = o3;
+    }
+}
+
 static bool all_aligned(size_t a, std::initializer_list<const void*> ps) {
     for (const void* p : ps)
         if (p && !aligned(p, a)) return false;
@@ -117,12 +173,19 @@ static plic_status launch_adjoint(const void* nx, const void* ny, const void* nz
                                   const void* g, void* gs, void* gx, void* gy, void* gz,
                                   int64_t n, void* stream) {
     const int vec_ok = all_aligned(16, {nx, ny, nz, d0, g, gs, gx, gy, gz});
-    const void* k = reinterpret_cast<const void*>(&k_plic_adjoint<T, MODE>);
     const int W = V16<T>::W;
-    const int grid = stream_grid(k, 256, vec_ok ? (n + W - 1) / W : n);
-    k_plic_adjoint<T, MODE><<<grid, 256, 0, as_stream(stream)>>>(
-        (const T*)nx, (const T*)ny, (const T*)nz, (const T*)d0, (const T*)g, (T*)gs, (T*)gx,
-        (T*)gy, (T*)gz, n, vec_ok);
+    const int64_t work = vec_ok ? (n + W - 1) / W : n;
+    if constexpr (W == 2) {
+        const int grid = stream_grid(reinterpret_cast<const void*>(&k_plic_adjoint64<MODE>), 256, work);
+        k_plic_adjoint64<MODE><<<grid, 256, 0, as_stream(stream)>>>(
+            (const fx::u64*)nx, (const fx::u64*)ny, (const fx::u64*)nz, (const fx::u64*)d0, (const T*)g, (T*)gs,
+            (T*)gx, (T*)gy, (T*)gz, n, vec_ok);
+    } else {
+        const int grid = stream_grid(reinterpret_cast<const void*>(&k_plic_adjoint<T, MODE>), 256, work);
+        k_plic_adjoint<T, MODE><<<grid, 256, 0, as_stream(stream)>>>(
+            (const T*)nx, (const T*)ny, (const T*)nz, (const T*)d0, (const T*)g, (T*)gs, (T*)gx, (T*)gy, (T*)gz, n,
+            vec_ok);
+    }
     return check_launch(MODE == 0 ? "plic_offset_backward" : "plic_volume_backward");
 }
 
