@@ -265,11 +265,13 @@ k_plic_offset_compact(const T* __restrict__ nx, const T* __restrict__ ny, const 
 // FP32 instructions: each thread takes 4 cells per step as two pairs, so every
 // cell sees identical arithmetic wherever it lies.  VEC (every array on a
 // 16-byte boundary): consecutive cells through one 16-byte load per array.
-// Otherwise (an odd row of a (3, n) tensor, a slice): cells 256 apart, each
-// array read in whole 128-byte lines of one warp, four loads per array in
-// flight.  The cells left over (n mod 4, n mod 1024) take one lane each, the cell in
-// both lanes of the pair; all unaligned cells that way took 88 us for 10 M cells
-// of the analytic solution, 39 us this way.
+// Otherwise (an odd row of a (3, n) tensor, a slice): cells 32 apart, a run of
+// 128 cells per warp, four loads per array in flight.  The cells left over (n mod 4, n
+// mod 1024) take one lane each, the cell in both lanes of the pair; all unaligned cells
+// that way took 88 us for 10 M cells of the analytic solution, 40 us this way (aligned
+// arrays: 35; 64 M: 222 and 193, with cells 256 apart 227, whose neighbouring warps
+// fetch the sector between their lines twice; 16-byte loads of the enclosing
+// vectors, shifted across the lanes: 249).
 // With ROUNDTRIP the forward volume of each stored d0 is written to vrt in
 // the same pass (plic_offset_roundtrip); COUNT (an invalid-cell counter was
 // given) keeps the per-cell count of invalid inputs, which otherwise costs
@@ -316,25 +318,25 @@ k_plic_offset_pair(const float* __restrict__ nx, const float* __restrict__ ny,
     } else {
         tail = n & ~(int64_t)1023;
         for (int64_t i0 = (int64_t)blockIdx.x * 1024; i0 < tail; i0 += 4 * stride) {
-            const int64_t i = i0 + threadIdx.x;
+            const int64_t i = i0 + ((threadIdx.x & ~31u) * 4u + (threadIdx.x & 31u));
             float a[4], b[4], c[4], v[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                a[j] = __ldcs(nx + i + 256 * j);
-                b[j] = __ldcs(ny + i + 256 * j);
-                c[j] = __ldcs(nz + i + 256 * j);
-                v[j] = __ldcs(V0 + i + 256 * j);
+                a[j] = __ldcs(nx + i + 32 * j);
+                b[j] = __ldcs(ny + i + 32 * j);
+                c[j] = __ldcs(nz + i + 32 * j);
+                v[j] = __ldcs(V0 + i + 32 * j);
             }
 #pragma unroll
             for (int j = 0; j < 4; j += 2) {
                 const float2 r = p2::offset_pair<METHOD, POLISH, ROUNDTRIP, COUNT>(
                     make_float2(a[j], a[j + 1]), make_float2(b[j], b[j + 1]), make_float2(c[j], c[j + 1]),
                     make_float2(v[j], v[j + 1]), bad, &w0);
-                __stcs(d0 + i + 256 * j, r.x);
-                __stcs(d0 + i + 256 * (j + 1), r.y);
+                __stcs(d0 + i + 32 * j, r.x);
+                __stcs(d0 + i + 32 * (j + 1), r.y);
                 if (ROUNDTRIP) {
-                    __stcs(vrt + i + 256 * j, w0.x);
-                    __stcs(vrt + i + 256 * (j + 1), w0.y);
+                    __stcs(vrt + i + 32 * j, w0.x);
+                    __stcs(vrt + i + 32 * (j + 1), w0.y);
                 }
             }
         }
