@@ -8,8 +8,10 @@
 // persistent wave).  Loads and the store are streaming (evict-first): every
 // byte is touched once.
 //
-// Roofline: 20 B/cell in FP32 (16 in, 4 out), 40 B/cell in FP64.  The FP32
-// solvers sit near the HBM/ALU balance point; FP64 is bound by the FP64 pipe.
+// Roofline: 20 B/cell in FP32 (16 in, 4 out), 40 B/cell in FP64.  The closed-form
+// FP32 solvers run at the HBM rate (k_plic_offset_pair); in FP64 the optimised SZ and
+// the analytic solution are bound by instruction issue (k_plic_offset_fx), the other
+// methods by the FP64 pipe.
 #include "host_common.h"
 #include "plic_fx.cuh"
 #include "plic_pair.cuh"
@@ -63,7 +65,8 @@ k_plic_offset(const T* __restrict__ nx, const T* __restrict__ ny, const T* __res
     count_invalid(bad, invalid);
 }
 
-// Work-compacted form of k_plic_offset for the default (non-literal) solvers:
+// Work-compacted form of k_plic_offset for the default (non-literal) forms of the
+// iterative solvers and, in FP64, of Kawano's SZ:
 // the warp runs the symmetry front end and the closed-form cases (Eqs. 24-25)
 // on its 32 x W cells, then gathers the cells that need the heavy part (the
 // trigonometric root of cases (3)/(4), or the Newton / nested-interval
@@ -116,14 +119,14 @@ k_plic_offset_compact(const T* __restrict__ nx, const T* __restrict__ ny, const 
                       unsigned long long* invalid, void* /* round trip: not fused here */) {
     typedef typename Vec16<T>::type VT;
     constexpr int W = Vec16<T>::W;
-    constexpr bool SZ = METHOD == M_SZ_ORIG || METHOD == M_SZ_OPT;
+    constexpr bool SZ = METHOD == M_SZ_ORIG;
     typedef Solver<METHOD, T, false> S;
     // FP64: one task list for the block's 8 warps (heavy parts long enough
     // to repay the barriers; only the block's last round is partly empty);
     // FP32: one list per warp, no barriers
     constexpr bool POOL = sizeof(T) == 8;
     // FP64: the front end on the bit patterns (front_bits), except for nested
-    // intervals (4-5 % faster for the other four solvers, 3 % slower there)
+    // intervals (4-5 % faster for the others, 3 % slower there)
     constexpr bool BITS = sizeof(T) == 8 && METHOD != M_NESTED;
     __shared__ T task[8][32 * W][4];
     __shared__ int wtot[8];
@@ -531,8 +534,7 @@ static const void* cptr() {
 // cosine on the FP32 pipes) is too short to repay the packing (measured 102
 // against 130 G solves/s one cell after the other, on 2^26 cells), and only
 // its faithful form reaches this function in FP32.  In FP64, and for the
-// iterative solvers, packing wins (e.g. nested intervals FP32 27 -> 40, FP64
-// SZ-opt 3.3 -> 4.5 G solves/s).
+// iterative solvers, packing wins (e.g. nested intervals FP32 27 -> 40 G solves/s).
 template <int METHOD>
 static const void* pick(plic_precision p, bool faithful, bool vec) {
     if constexpr (METHOD == M_SZ_OPT || METHOD == M_ANALYTIC) {
@@ -543,15 +545,15 @@ static const void* pick(plic_precision p, bool faithful, bool vec) {
         return p == PLIC_FP64 ? kptr<METHOD, double, false, true>()
              : p == PLIC_FP32_POLISHED ? kptr<METHOD, float, true, true>() : kptr<METHOD, float, false, true>();
     } else {
-    if (p == PLIC_FP64_REFINED) return reinterpret_cast<const void*>(&k_plic_offset_refined<METHOD>);
-    if (p == PLIC_FP64)
-        return faithful ? kptr<METHOD, double, false, true>() : cptr<METHOD, double, false>();
-    const bool compact = !faithful && METHOD != M_SZ_ORIG;
-    if (p == PLIC_FP32_POLISHED)
-        return compact ? cptr<METHOD, float, true>()
-                      : (faithful ? kptr<METHOD, float, true, true>() : kptr<METHOD, float, true, false>());
-    return compact ? cptr<METHOD, float, false>()
-                  : (faithful ? kptr<METHOD, float, false, true>() : kptr<METHOD, float, false, false>());
+        if (p == PLIC_FP64_REFINED) return reinterpret_cast<const void*>(&k_plic_offset_refined<METHOD>);
+        if (p == PLIC_FP64)
+            return faithful ? kptr<METHOD, double, false, true>() : cptr<METHOD, double, false>();
+        if constexpr (METHOD == M_SZ_ORIG)           // its default form is paired (pick_pair)
+            return p == PLIC_FP32_POLISHED ? kptr<METHOD, float, true, true>() : kptr<METHOD, float, false, true>();
+        else if (p == PLIC_FP32_POLISHED)
+            return faithful ? kptr<METHOD, float, true, true>() : cptr<METHOD, float, true>();
+        else
+            return faithful ? kptr<METHOD, float, false, true>() : cptr<METHOD, float, false>();
     }
 }
 

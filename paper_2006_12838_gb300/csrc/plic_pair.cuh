@@ -57,26 +57,6 @@ __device__ __forceinline__ f2 sqrtp(f2 x) {
     return mul(x, rsqrt(x));
 }
 
-// arcsine on [0, 1], two lanes at once: asin(s) = s + s^3 P(s^2) on
-// s <= 1/2 with P a degree-4 least-squares fit to (asin(s) - s)/s^3 on
-// [0, 1/4] (relative error below 2e-8, under the FP32 rounding), and the
-// half-angle reduction asin(a) = pi/2 - 2 asin(sqrt((1 - a)/2)) above 1/2.
-// The optimised-SZ argument is never negative: it is 1.5 n1 n2 (n1+n2-2 n3 V)/t^3
-// with n1+n2 > 2 n3 V outside case (5), or 0.75 n1 n2 n3 (1-2V)/t^3 with V <= 1/2.
-__device__ __forceinline__ f2 asin01(f2 a) {
-    const b2 big = lt(mk(0.5f), a);
-    const f2 zb = mul(mk(0.5f), sub(mk(1.0f), a));
-    const f2 z = sel(big, zb, mul(a, a));
-    const f2 s = sel(big, sqrtp(z), a);
-    f2 p = mk(0.038206491619348526f);
-    p = fma(p, z, mk(0.026494324207305908f));
-    p = fma(p, z, mk(0.045010678470134735f));
-    p = fma(p, z, mk(0.07498809695243835f));
-    p = fma(p, z, mk(0.16666673123836517f));
-    p = fma(mul(s, z), p, s);
-    return sel(big, fma(mk(-2.0f), p, mk(1.5707963267948966f)), p);
-}
-
 // One Newton step on the cubic of Eq. 10 for cases (3)/(4) (d >= n2, n1 > 0),
 // with g and g' multiplied through by n1 so that one reciprocal serves:
 // n1 g = n1 (3 d (d - n1) + n1^2) - (d - n2)^3 - (d - n3)_+^3 - 6 n1 n2 n3 V,
@@ -95,7 +75,7 @@ __device__ __forceinline__ f2 polish34(f2 d, f2 V6, f2 n1, f2 n2, f2 n3) {
 }
 
 // The smaller positive root w of the depressed cubic w^3 - Q w + R = 0 of cases
-// (3)/(4), from nQ = -Q < 0 and R >= 0 (sz_opt below).  Viete's form is
+// (3)/(4), from nQ = -Q < 0 and R >= 0 (centre_distance below).  Viete's form is
 // w = 2 t sin(asin(a)/3) with t^2 = Q/3, a = R/(2 t^3); in these cases
 // a <= 0.8839, clear of the arcsine's singular end, so one odd polynomial (an
 // equal-ripple fit of 2 sin(asin(a)/3) on a <= 0.886, degree 9, within 8e-5)

@@ -354,39 +354,6 @@ __device__ __forceinline__ T solve_sz_opt(T V, T n1, T n2, T n3) {
     return solve_sz_opt_default<T, !FAITHFUL>(V, n1, n2, n3);
 }
 
-// The two parts of the optimised SZ solution (the FP64 path branches on the
-// cases; the FP32 path selects and has its own paired kernel).
-template <typename T, bool FAITHFUL>
-__device__ __forceinline__ bool sz_opt_easy(T V, T n1, T n2, T n3, T& d) {
-    typedef Fm<T> F;
-    typedef Kc<T> K;
-    const T n12 = n1 + n2, n3V = n3 * V;
-    const T V6n2n3 = T(6) * n2 * n3V, sqn1 = n1 * n1;
-    if (n12 <= T(2) * n3V) { d = n3V + T(0.5) * n12; return true; }
-    if (V6n2n3 < sqn1) { d = F::cbrt_(V6n2n3 * n1); return true; }
-    if (T(3) * n2 * (T(2) * n3V + n1 - n2) < sqn1) {
-        d = T(0.5) * (n1 + F::sqrt_(T(8) * n2 * n3V - K::third * sqn1));
-        return true;
-    }
-    return false;
-}
-
-template <typename T, bool FAITHFUL>
-__device__ __forceinline__ T sz_opt_hard(T V, T n1, T n2, T n3) {
-    typedef Fm<T> F;
-    typedef Kc<T> K;
-    const T n12 = n1 + n2, n3V = n3 * V, n1n2 = n1 * n2;
-    const T num3 = sq(n3) * (T(3) * n12 - n3) + n1 * n1 * (n1 - T(3) * n3) + sq(n2) * (n2 - T(3) * n3);
-    const bool c3 = !(n3 < n12) || T(6) * n2 * n3V * n1 < num3;
-    const T q = c3 ? T(1.5) * n1n2 * (n12 - T(2) * n3V) : T(0.75) * n1n2 * n3 * (T(1) - T(2) * V);
-    const T t2 = c3 ? T(2) * n1n2 : T(0.25) * (n1 * (T(2) * (n2 + n3) - n1) - sq(n3 - n2));
-    const T c = c3 ? n12 : T(0.5);
-    const T rt = F::rsqrt_(t2);
-    T arg = q * (rt * rt * rt);
-    if (!FAITHFUL) arg = fmin(fmax(arg, T(-1)), T(1));
-    return c - T(2) * (t2 * rt) * F::sin_pi6_(K::third * F::asin_(arg));
-}
-
 // ----------------------------------------------------------------------------
 // Sec. 2.5: the iterative solvers.  Both take the closed forms for cases (5)
 // and (2), then iterate on the volume of Eq. 10 inside the bracket of a case:
@@ -548,20 +515,12 @@ __device__ __forceinline__ T solve_nested(T V, T n1, T n2, T n3) {
     return nested_easy<T, FAITHFUL>(V, n1, n2, n3, d) ? d : nested_hard<T, FAITHFUL>(V, n1, n2, n3);
 }
 
-// The split parts by method, for the work-compacted kernel (reduced inputs:
-// the L1-normalised m for the SZ solutions, the unit-normal n otherwise).
+// The split parts by method, for the work-compacted kernel (reduced inputs: the
+// L1-normalised m for Kawano's SZ solution, the unit-normal n otherwise).
 template <int METHOD, typename T, bool FAITHFUL> struct Solver;
-template <typename T, bool F> struct Solver<M_ANALYTIC, T, F> {
-    static __device__ __forceinline__ bool easy(T V, T a, T b, T c, T& d) { return analytic_easy<T, F>(V, a, b, c, d); }
-    static __device__ __forceinline__ T hard(T V, T a, T b, T c) { return analytic_hard<T, F>(V, a, b, c); }
-};
 template <typename T, bool F> struct Solver<M_SZ_ORIG, T, F> {
     static __device__ __forceinline__ bool easy(T V, T a, T b, T c, T& d) { return sz_orig_easy<T, F>(V, a, b, c, d); }
     static __device__ __forceinline__ T hard(T V, T a, T b, T c) { return sz_orig_hard<T, F>(V, a, b, c); }
-};
-template <typename T, bool F> struct Solver<M_SZ_OPT, T, F> {
-    static __device__ __forceinline__ bool easy(T V, T a, T b, T c, T& d) { return sz_opt_easy<T, F>(V, a, b, c, d); }
-    static __device__ __forceinline__ T hard(T V, T a, T b, T c) { return sz_opt_hard<T, F>(V, a, b, c); }
 };
 template <typename T, bool F> struct Solver<M_NEWTON, T, F> {
     static __device__ __forceinline__ bool easy(T V, T a, T b, T c, T& d) { return newton_easy<T, F>(V, a, b, c, d); }
@@ -608,7 +567,8 @@ __device__ __forceinline__ T offset_cell(T nx, T ny, T nz, T V0, int& bad) {
 }
 
 // ----------------------------------------------------------------------------
-// FP64 result from an FP32 solve, without the FP64 pipe (PLIC_FP64_REFINED).
+// FP64 result from an FP32 solve, without the FP64 pipe (PLIC_FP64_REFINED; the
+// optimised SZ and the analytic solution: plic_fx.cuh).
 // The doubles are split into double-floats (hi + lo, 48 significant bits) by
 // integer operations; the symmetry reduction (Eqs. 2-8) sorts |n| on the bit
 // patterns and forms V = min(V0, 1 - V0) from the bits (1 - V0 as an exact
@@ -662,19 +622,17 @@ __device__ __forceinline__ double offset_cell_refined(double nx, double ny, doub
     const float Vf = V.hi;
     // FP32 solve of the reduced problem, as an offset d from the corner
     df d;
-    if (METHOD == M_SZ_ORIG || METHOD == M_SZ_OPT) {
+    if (METHOD == M_SZ_ORIG) {
         const float il = Fm<float>::rcp_(L.hi);
         const float m1 = n1.hi * il, m3 = n3.hi * il;
         const float m2 = Fm<float>::fdim_(1.0f, m1 + m3);
-        float a = METHOD == M_SZ_ORIG ? solve_sz_orig<float, false>(Vf, m1, m2, m3)
-                                      : solve_sz_opt<float, false>(Vf, m1, m2, m3);
+        float a = solve_sz_orig<float, false>(Vf, m1, m2, m3);
         a = polish<float>(a, Vf, m1, m2, m3);
         if (a != a) return __longlong_as_double(0x7FF8000000000000ll);  // Kawano's NaN
         d = df_mul_f(L, a);
     } else {
-        float e = METHOD == M_ANALYTIC ? solve_analytic<float, false>(Vf, n1.hi, n2.hi, n3.hi)
-                : METHOD == M_NEWTON   ? solve_newton<float, false>(Vf, n1.hi, n2.hi, n3.hi)
-                                       : solve_nested<float, false>(Vf, n1.hi, n2.hi, n3.hi);
+        float e = METHOD == M_NEWTON ? solve_newton<float, false>(Vf, n1.hi, n2.hi, n3.hi)
+                                     : solve_nested<float, false>(Vf, n1.hi, n2.hi, n3.hi);
         e = polish<float>(e, Vf, n1.hi, n2.hi, n3.hi);
         if (e != e) return __longlong_as_double(0x7FF8000000000000ll);
         d = df_make(e);
