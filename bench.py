@@ -161,11 +161,13 @@ class ClockSampler:
 # * closed forms: case (5) 1, case (2) 3 + sqrt, case (1) 1 + cbrt;
 # * FP32-polished: the Newton step on Eq. 10 for cases (1)-(4), 22 + 2 div
 #   (2 in case (5));
-# * analytic, cases (3)/(4): the case test from the residual at d = n3
-#   (21 + div), the coefficients (11 in case (3), 15 in case (4)) and the root
-#   of Eq. 11 (10 + cbrt, rsqrt, sqrt, atan2, sin);
-# * optimised SZ: 28 for the division-free case tests, then 1 / 3 + sqrt /
-#   1 + cbrt for cases (5) / (2) / (1), or 18 + rsqrt, asin, sin for (3)/(4);
+# * optimised SZ and analytic in FP32 (p2::centre_distance; both precisions are
+#   one kernel): the common products and the test of case (5) 6 and its offset
+#   2; the test of cases (1)/(2) 6, then 5 + cbrt / 8 + sqrt; cases (3)/(4) the
+#   case test 7, the coefficients 2 / 6, the root of the depressed cubic 17 +
+#   rsqrt + div (polynomial start and one Newton step) and 2 for the offset;
+# * the same two in FP64 and FP64_REFINED (plic_fx.cuh): 6 FP64 operations per cell;
+#   the rest runs on the integer and FP32 pipes, for which there is no probe;
 # * Kawano's SZ: its thresholds (10 + 2 div; 16 + 2 div more where cases
 #   (3)-(5) are told apart), the closed forms, and for (3)/(4) Viete's root
 #   (12 + sqrt, div, acos, cos);
@@ -189,6 +191,10 @@ class ClockSampler:
 FE, FE_L1 = 18, 4
 CLASSIFY = 14
 CLOSED = {5: (1, {}), 2: (3, {"sqrt": 1}), 1: (1, {"cbrt": 1})}
+CENTRE = ("sz_opt", "analytic")
+CENTRE_COST = {5: (8, {}), 1: (17, {"cbrt": 1}), 2: (20, {"sqrt": 1}), 3: (40, {"rsqrt": 1, "div": 1}),
+               4: (44, {"rsqrt": 1, "div": 1})}
+CENTRE_FP64 = 6
 POLISH = (22, {"div": 2})
 POLISH5 = (2, {})
 NEWTON_STEPS = {1: 7, 3: 4, 4: 4}
@@ -216,23 +222,14 @@ def ops_per_case(method: str, prec: str):
         base = (FE, {})
         if method in ("sz_opt", "sz_orig"):
             base = _add(base, (FE_L1, {"div": 1}))
-        if method == "sz_opt":
-            cost = (28, {})
-            cost = _add(cost, CLOSED[c] if c in CLOSED else (18, {"rsqrt": 1, "asin": 1, "sin": 1}))
+        if method in CENTRE:
+            cost = CENTRE_COST[c]
         elif method == "sz_orig":
             cost = (10, {"div": 2})
             if c in (3, 4, 5):
                 cost = _add(cost, (16, {"div": 2}))
             cost = _add(cost, CLOSED[c] if c in CLOSED else
                         (12, {"sqrt": 1, "div": 1, "acos": 1, "cos": 1}))
-        elif method == "analytic":
-            cost = (CLASSIFY, {})
-            if c in CLOSED:
-                cost = _add(cost, CLOSED[c])
-            else:
-                cost = _add(cost, (21, {"div": 1}))
-                cost = _add(cost, (11 if c == 3 else 15, {}))
-                cost = _add(cost, (10, {"cbrt": 1, "rsqrt": 1, "sqrt": 1, "atan2": 1, "sin": 1}))
         elif method == "newton":
             cost = (CLASSIFY, {})
             if c in (5, 2):
@@ -251,7 +248,7 @@ def ops_per_case(method: str, prec: str):
         else:
             raise ValueError(method)
         tot = _add(base, cost)
-        if prec == "fp32p":
+        if prec == "fp32p" and method not in CENTRE:
             tot = _add(tot, POLISH5 if c == 5 else POLISH)
         out[c] = tot
     return out
@@ -282,6 +279,8 @@ def fp32_pipes(method: str, prec: str, hist):
 def fp64_equivalents(method: str, hist, call_cost):
     """FP64-FMA equivalents per cell: the operations plus each library call
     at its measured cost (``call_cost``: {call: FMA equivalents})."""
+    if method in CENTRE:
+        return CENTRE_FP64
     ops, calls = ops_weighted(method, "fp64", hist)
     return ops + sum(v * call_cost[k] for k, v in calls.items())
 
@@ -474,13 +473,13 @@ def op_roofline(sec_per_cell, bytes_per_cell, pk, pp, fp32=0.0, mufu=0.0, fp64=0
 #   per cell: stencil sums 54, interface tests 52, normal 10, frame 19,
 #     per-normal solver constants 72, LDL^T factor 55 + solve 25, Eq. 42 12 -> 299
 #     (MUFU 20: normal 2, frame 1, constants 11, pivots 5, Eq. 42 1)
-#   per PLIC solve (m + 1 of them): 59 (MUFU 6: sqrt, cube root 2, arcsine, sine,
-#     polish reciprocal)
+#   per PLIC solve (m + 1 of them): 32 (MUFU 4: sqrt, cube root 2, the root's
+#     reciprocal)
 #   per neighbour: foot point 11, normal equations 23                     -> 34
 # The peaks are the unit counts times the maximum SM clock: 128 FP32 lanes and
 # 16 MUFU lanes per SM, 152 SMs.
-CURV_FP_CELL, CURV_FP_SOLVE, CURV_FP_NEIGHBOUR = 299, 59, 34
-CURV_XU_CELL, CURV_XU_SOLVE = 20, 6
+CURV_FP_CELL, CURV_FP_SOLVE, CURV_FP_NEIGHBOUR = 299, 32, 34
+CURV_XU_CELL, CURV_XU_SOLVE = 20, 4
 N_SM, FP32_PER_SM, XU_PER_SM = 152, 128, 16
 
 
@@ -558,7 +557,7 @@ def section_solvers(t32, dev, pk, steps, hist=None, pp=None):
     return out
 
 
-# FP64_REFINED adds to the FP32-polished solve two Newton steps on Eq. 10 in
+# FP64_REFINED (Kawano, Newton, nested) adds to the FP32-polished solve two Newton steps on Eq. 10 in
 # double-float arithmetic (about 8 double-float products at ~10 FP32
 # operations and 8 sums at ~15 per step) and the integer front end on the
 # doubles' bits (~60): an estimate of 460 FP32/ALU operations per cell.
@@ -580,7 +579,7 @@ def section_fp64(dev, pk, steps, cells, hist=None, pp=None, samples=None):
                  "hbm_frac": frac(gbs, pk["hbm_gbs"]), "cells": cells}
             if hist and pp:
                 spc = sec / steps / cells
-                if prec == "fp64":
+                if prec == "fp64" or m in CENTRE:
                     eq = fp64_equivalents(m, hist, pp["fp64_call_fma_equiv"])
                     r["roofline"] = op_roofline(spc, 40.0, pk, pp, fp64=eq)
                 else:
@@ -1003,8 +1002,7 @@ def run_case(args):
             plic.curvature(phi, idx[:k].contiguous())
     elif args.case == "compact":
         # the 256^3 curvature field tiled to nz, ny, nx = 256, 256, 1024 (256 MiB,
-        # twice L2): rows of 1024 cells (the count pass's 512-cell segments) and
-        # 8192 tiles (the scan launch)
+        # twice L2): 8192 tiles of 8192 cells
         phi, _ = synth.curvature_field(seed=3, edge=256, device=dev)
         big = phi.repeat(1, 1, 4)
         idx = torch.empty(big.numel() // 8, dtype=torch.int32, device=dev)

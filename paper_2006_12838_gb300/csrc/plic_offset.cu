@@ -373,11 +373,11 @@ __device__ __noinline__ double offset_cell_slow(double nx, double ny, double nz,
 // stores its own cells.  The arrays are read as integers: of the bits of a double in
 // a register the compiler makes |x| an operation on the FP64 pipe (three per cell:
 // 396 against 317 us).
-// Bound: integer issue (443 warp instructions per 32 cells, ALU pipe 60 % busy)
-// beside the FP64 pipe (7 instructions).  2^24 cells: closed forms 3200 us (optimised
+// Bound: instruction issue (477 warp instructions per 32 cells, 72 % of the slots; ALU
+// pipe 68 % busy) beside the FP64 pipe (7 instructions, 67 %).  2^24 cells: closed forms 3200 us (optimised
 // SZ, FP64 pipe 85 % busy) and 4490 us (analytic); this scheme with one thread running
 // each of its cells through its case 379 us (every case of the warp in turn, 18.8 lanes
-// on) and with the tests in fixed point too; packed 285 us (28.4 lanes on).  16 M
+// on) and with the tests in fixed point too; packed 284 us (27 lanes on).  16 M
 // cells FP64_REFINED 555 (double-float steps) -> 273 us.  256 threads and 1024 cells per
 // block 295 us, 64 and 256 295 us; ten blocks per SM (48 registers) 285, eight 287 us.
 // Below 2^15 cells 8.2 us at any shape (closed forms 18-22 us).
