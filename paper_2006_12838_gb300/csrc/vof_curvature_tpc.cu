@@ -9,12 +9,12 @@
 // instruction count decides instead, and one thread per cell does each step
 // once:
 //   - the 27 stencil values with compile-time offsets, the Parker-Youngs (or
-//     centre-of-mass) sums and the interface mask in registers;
+//     centre-of-mass) sums in registers and the list of the interface neighbours in
+//     shared memory;
 //   - normal, frame, centre offset d0(phi_0, n) and the per-normal constants
 //     of the solver once;
-//   - a loop over the set bits of the mask only (the interface neighbours of
-//     Eq. 36), two neighbours per trip: their values come back from the
-//     thread's column in shared memory, their offsets are solved together (paired FP32
+//   - a loop over that list only (Eq. 36), two neighbours per trip: their
+//     offsets are solved together (paired FP32
 //     instructions for the optimised SZ solution), their points accumulated
 //     into the normal equations in registers;
 //   - the 5x5 solve of the fit precision and Eq. 42, as in the lane phase of
@@ -28,24 +28,25 @@
 namespace plic {
 
 // kappa (sign per flags) of interface cell c of a field, one thread.  sv: the
-// thread's column of 27 values in shared memory, TPC_THREADS apart: the stencil's
-// values as the prologue reads them, from where the loop takes those of its
-// neighbours (one word per lane and bank; read from the field again they cost a 16-byte
-// table read of the integer direction, the address arithmetic and a load of five or
-// six wavefronts: batch of 64 fields, 2.6 M cells, 216 -> 200 us, 1 GiB field with its
-// compaction 215 -> 212).
+// thread's column of 28 entries in shared memory, TPC_THREADS apart.  The prologue
+// lists the interface neighbours there as it reads them, each with its value and the
+// byte offset of its direction in tab.ef (one 8-byte word per lane, conflict-free), and
+// the loop takes two entries per trip.  Reading each value from the field again through
+// a table of integer directions cost the address arithmetic and a load of five or six
+// wavefronts: batch of 64 fields, 2.6 M cells, 216.5 us; all 27 values in the
+// column and the neighbours from the bits of a mask 200.3; this list 198.1 (1 GiB
+// field with its compaction 215.5 -> 212).
 template <int METHOD, int FIT>
 __device__ __forceinline__ float tpc_kappa(const float* __restrict__ phi, int nx, int64_t nxy,
-                                           int64_t c, uint32_t flags, const E27Shared& tab, float* sv) {
+                                           int64_t c, uint32_t flags, const E27Shared& tab, float2* sv) {
     const bool cm = (flags & PLIC_FLAG_NORMAL_CM) != 0;
     const float* p0 = phi + c;
     // offsets within the field in 32 bits (list entries are int32 cell indices)
     const int nxy32 = (int)nxy;
-    // 1. stencil: normal sums (Eq. 38 weights or all 1) and interface mask
+    // 1. stencil: normal sums (Eq. 38 weights or all 1) and the interface neighbours
     float gx = 0.0f, gy = 0.0f, gz = 0.0f;
-    unsigned mask = 0u;
     const float phi0 = __ldg(p0);
-    sv[0] = phi0;
+    float2* tail = sv;
     for_e27<1>([&](auto I) {
         constexpr int i = decltype(I)::value;
         constexpr int p = E27Table::v[i];
@@ -53,14 +54,16 @@ __device__ __forceinline__ float tpc_kappa(const float* __restrict__ phi, int nx
         constexpr int e2 = ex * ex + ey * ey + ez * ez;
         constexpr float wpy = e2 == 1 ? 4.0f : (e2 == 2 ? 2.0f : 1.0f);
         const float v = __ldg(p0 + (ex + ey * nx + ez * nxy32));
-        sv[i * TPC_THREADS] = v;
         const float w = cm ? 1.0f : wpy;
         if (ex != 0) gx = fmaf(w * (float)ex, v, gx);
         if (ey != 0) gy = fmaf(w * (float)ey, v, gy);
         if (ez != 0) gz = fmaf(w * (float)ez, v, gz);
         // 0 < v < 1 as one unsigned compare of the bits: the positive floats
         // below 1.0f are the patterns 1 .. 0x3F7FFFFF
-        if (__float_as_uint(v) - 1u < 0x3F7FFFFFu) mask |= 1u << i;
+        if (__float_as_uint(v) - 1u < 0x3F7FFFFFu) {
+            *tail = make_float2(v, __int_as_float((int)sizeof(float4) * i));
+            tail += TPC_THREADS;
+        }
     });
     // 2. normal and frame (Sec. 4.2)
     const float gl2 = gx * gx + gy * gy + gz * gz;
@@ -92,19 +95,17 @@ __device__ __forceinline__ float tpc_kappa(const float* __restrict__ phi, int nx
     float rec[21];
 #pragma unroll
     for (int q = 0; q < 20; ++q) rec[q] = 0.0f;
-    rec[20] = (float)__popc(mask);
+    rec[20] = (float)((int)(tail - sv) / TPC_THREADS);
+    *tail = make_float2(phi0, __int_as_float(0));
     // two neighbours per trip (in ascending order; an odd last one pairs with
-    // the centre, the zero point of the list, which adds nothing)
-    unsigned list = mask;
+    // the centre, the zero point behind the list, which adds nothing)
 #pragma unroll 1
-    while (list) {
-        const int i1 = __ffs(list) - 1;
-        list &= list - 1u;
-        const int i2 = list != 0u ? __ffs(list) - 1 : 0;
-        list &= list - 1u;                          // no-op on an empty list
-        const float4 f1 = tab.ef[i1], f2 = tab.ef[i2];
-        const float v1 = sv[i1 * TPC_THREADS], v2 = sv[i2 * TPC_THREADS];
-        const p2::f2 d0i = offset_two<METHOD>(pl, make_float2(v1, v2));
+    for (const float2* r = sv; r < tail; r += 2 * TPC_THREADS) {
+        const float2 r1 = r[0], r2 = r[TPC_THREADS];
+        const int i1 = __float_as_int(r1.y), i2 = __float_as_int(r2.y);
+        const float4 f1 = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(tab.ef) + i1);
+        const float4 f2 = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(tab.ef) + i2);
+        const p2::f2 d0i = offset_two<METHOD>(pl, make_float2(r1.x, r2.x));
         float qx[2] = {f1.x, f2.x}, qy[2] = {f1.y, f2.y};
         float qz[2] = {f1.z, f2.z}, z[2];
         const float dd[2] = {d0i.x, d0i.y};
@@ -158,7 +159,7 @@ k_vof_curvature_tpc(const float* __restrict__ phi, int nx, int ny, const int32_t
         lim = dn < n ? dn : n;
     }
     __shared__ E27Shared tab;
-    __shared__ float sv[27 * TPC_THREADS];
+    __shared__ float2 sv[28 * TPC_THREADS];
     tab.fill();
     const int64_t nxy = (int64_t)nx * ny;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < lim;
@@ -176,7 +177,7 @@ k_vof_curvature_batched_tpc(const vof_field* __restrict__ fields, const int64_t*
                             unsigned long long* __restrict__ ticket, uint32_t flags) {
     const int lane = threadIdx.x & 31;
     __shared__ E27Shared tab;
-    __shared__ float sv[27 * TPC_THREADS];
+    __shared__ float2 sv[28 * TPC_THREADS];
     tab.fill();
     pdl_wait();                  // the tables are written
     for (;;) {
