@@ -190,7 +190,7 @@ extern "C" plic_status vof_curvature_batched(const vof_field* fields, int n_fiel
     if (!fields || !workspace) return PLIC_ERR_ARG;
     if (ws_bytes < plic_workspace_bytes(PLIC_WS_BATCHED, n_fields)) return PLIC_ERR_ARG;
     if (!aligned(workspace, 256)) return PLIC_ERR_ALIGN;
-    int threads = CO_THREADS, chunk = 128, bps = 0, lanes = 0;
+    int threads = CO_THREADS, chunk = 0, bps = 0, lanes = 0;
     if (tuning) {
         threads = tuning->block_threads;
         chunk = tuning->cells_per_chunk;
@@ -202,7 +202,6 @@ extern "C" plic_status vof_curvature_batched(const vof_field* fields, int n_fiel
         if (threads != CO_THREADS) return PLIC_ERR_UNSUPPORTED;   // built for 4 warps per block
     }
     if (lanes == 0) lanes = BATCHED_DEFAULT_LANES;
-    chunk = (chunk + CO_BATCH - 1) / CO_BATCH * CO_BATCH;     // whole warp batches
     // argument checks and the total of the list lengths
     const size_t nf = (size_t)n_fields;
     int64_t total = 0;
@@ -216,6 +215,18 @@ extern "C" plic_status vof_curvature_batched(const vof_field* fields, int n_fiel
         total += F.n_iface;
     }
     if (total == 0) return PLIC_OK;
+    const void* k = lanes == 1 ? select_tpc(true, m, fit_mode(flags)) : select_coop(m, fit_mode(flags));
+    if (!k) return PLIC_ERR_ARG;
+    const int occ = blocks_per_sm(k, threads, 0);
+    const int per_sm = bps > 0 ? (bps < occ ? bps : occ) : occ;
+    int64_t grid = (int64_t)sm_count() * per_sm;
+    // Cells per ticket when the tuning leaves them open: 128, or as few as 32 where
+    // the resident warps would get fewer than four tickets each, since the last ones
+    // then set the time (0.4 M cells 43.6 us with 128, 37.6 with 32; 1.2 M cells 99 with
+    // 128 or 64, 101 with 32; 2.7 M cells 228 and 238).
+    if (chunk == 0)
+        for (chunk = 128; chunk > CO_BATCH && total < 4 * chunk * grid * CO_WARPS;) chunk /= 2;
+    chunk = (chunk + CO_BATCH - 1) / CO_BATCH * CO_BATCH;     // whole warp batches
     char* ws = reinterpret_cast<char*>(workspace);
     vof_field* d_fields = reinterpret_cast<vof_field*>(ws);
     const size_t off_pre = (nf * sizeof(vof_field) + 255) / 256 * 256;
@@ -238,11 +249,6 @@ extern "C" plic_status vof_curvature_batched(const vof_field* fields, int n_fiel
         e = cudaLaunchKernel(reinterpret_cast<const void*>(&k_batch_table), dim3(1), dim3(TABLE_FIELDS), targs, 0, s);
     }
     if (e != cudaSuccess) { set_last_error("vof_curvature_batched", e); return PLIC_ERR_CUDA; }
-    const void* k = lanes == 1 ? select_tpc(true, m, fit_mode(flags)) : select_coop(m, fit_mode(flags));
-    if (!k) return PLIC_ERR_ARG;
-    const int occ = blocks_per_sm(k, threads, 0);
-    const int per_sm = bps > 0 ? (bps < occ ? bps : occ) : occ;
-    int64_t grid = (int64_t)sm_count() * per_sm;
     const int64_t need = ((total + chunk - 1) / chunk + CO_WARPS - 1) / CO_WARPS;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;

@@ -55,3 +55,19 @@ def test_tables_and_capture(n):
         torch.cuda.synchronize()
         check()
     del junk, ws
+
+
+@pytest.mark.parametrize("copies", [1, 30, 60, 120])
+def test_ticket_sizes(copies):
+    """The cells per ticket chosen by the total (32, 64, 128) against fixed ones: the
+    same bits, from less than one ticket per warp up to several."""
+    dev = torch.device("cuda:0")
+    z, y, x = torch.meshgrid(*(torch.arange(96, device=dev, dtype=torch.float32),) * 3, indexing="ij")
+    phi = (40.0 - torch.sqrt((x - 47.3) ** 2 + (y - 48.1) ** 2 + (z - 46.9) ** 2) + 0.5).clamp(0, 1)
+    idx, cnt = plic.interface_compact(phi)
+    k = int(cnt.item())
+    want = plic.curvature(phi, idx, n_iface=k)
+    for tuning in (None, (128, 32, 0, 1), (128, 128, 0, 1)):
+        kappas = torch.full((copies, k), 7.0, device=dev)
+        plic.curvature_batched([(phi, idx, k, kappas[i]) for i in range(copies)], tuning=tuning)
+        assert torch.equal(kappas, want.expand(copies, k))
