@@ -293,7 +293,8 @@ typedef struct {
  * blocks).  `fields` is a HOST array of n_fields descriptors; they go to the
  * workspace by value (as kernel arguments, so a captured call keeps them) and
  * the array may be reused once the call returns.
- * tuning: nullable (defaults are used).  workspace: >=
+ * tuning: nullable (one thread per cell, chunks of 32 to 128 cells by the
+ * total).  workspace: >=
  * plic_workspace_bytes(PLIC_WS_BATCHED, n_fields) bytes, 256-byte aligned. */
 plic_status vof_curvature_batched(const vof_field *fields, int n_fields,
                                   const vof_tuning *tuning, plic_method m, uint32_t flags,
