@@ -32,6 +32,7 @@
 #include <stdio.h>
 
 #include "host_common.h"
+#include "workspace.h"
 
 namespace plic {
 
@@ -456,11 +457,7 @@ extern "C" size_t plic_workspace_bytes(int op, int64_t arg) {
             const size_t b = ((size_t)(arg / 16 + 1) * sizeof(unsigned) + 255) / 256 * 256;
             return a + b;
         }
-        case PLIC_WS_BATCHED: {
-            // descriptor table + per-field cell prefix + the ticket counter
-            const size_t b = (size_t)arg * (sizeof(vof_field) + sizeof(int64_t)) + 2 * sizeof(int64_t);
-            return (b + 255) / 256 * 256 + 256;
-        }
+        case PLIC_WS_BATCHED: return plic::batch_workspace((size_t)arg);
         default: return 0;
     }
 }

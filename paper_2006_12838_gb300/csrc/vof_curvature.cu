@@ -12,6 +12,7 @@
 // list length, so that a cell's kappa does not depend on the list (or the
 // buffer) it comes in.
 #include "host_common.h"
+#include "workspace.h"
 #include "vof_curvature_coop.cuh"
 
 namespace plic {
@@ -228,11 +229,10 @@ extern "C" plic_status vof_curvature_batched(const vof_field* fields, int n_fiel
         for (chunk = 128; chunk > CO_BATCH && total < 4 * chunk * grid * CO_WARPS;) chunk /= 2;
     chunk = (chunk + CO_BATCH - 1) / CO_BATCH * CO_BATCH;     // whole warp batches
     char* ws = reinterpret_cast<char*>(workspace);
+    const BatchLayout at = batch_layout(nf);
     vof_field* d_fields = reinterpret_cast<vof_field*>(ws);
-    const size_t off_pre = (nf * sizeof(vof_field) + 255) / 256 * 256;
-    int64_t* d_pre = reinterpret_cast<int64_t*>(ws + off_pre);
-    const size_t off_tk = off_pre + ((nf + 1) * sizeof(int64_t) + 255) / 256 * 256;
-    unsigned long long* d_ticket = reinterpret_cast<unsigned long long*>(ws + off_tk);
+    int64_t* d_pre = reinterpret_cast<int64_t*>(ws + at.prefix);
+    unsigned long long* d_ticket = reinterpret_cast<unsigned long long*>(ws + at.ticket);
     cudaStream_t s = as_stream(stream);
     cudaError_t e = cudaSuccess;
     int64_t before = 0;
