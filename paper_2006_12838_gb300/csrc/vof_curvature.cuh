@@ -322,8 +322,10 @@ struct UnitRoot {
 // volume, four threshold tests on V, the closed forms of cases (5), (2), (1)
 // (the last as cbrt(6 m1 m2 m3) * cbrt(V)), and the root of the depressed cubic
 // of cases (3)/(4) in units of t, whose argument a is linear in V: k3 V + a3 or
-// k4 V + a4 (p2::centre_distance; a clamped where the thresholds' rounding
-// lets a normal with m1 < 1e-14 m2 in).  All as distances s = 1/2 - d from the
+// k4 V + a4 (p2::centre_distance).  Where m1 < 1e-14 m2 the thresholds' rounding lets
+// volumes of cases (2) and (5) in, for which a is the difference of two large numbers,
+// of either sign; t is then below 1e-7, and any a in [0, 1] (saturated) gives their
+// offset to rounding.  All as distances s = 1/2 - d from the
 // cell's centre.  The thresholds are the product-form tests of
 // solve_sz_opt_default divided through once.
 template <>
@@ -377,7 +379,7 @@ struct CellPlic<M_SZ_OPT> {
     __device__ __forceinline__ float offset(float V0) const {
         const float V = fminf(V0, 1.0f - V0);
         const bool c3 = V < V3;
-        float s = fmaf(c3 ? t3 : t4, UnitRoot::eval(fminf(fmaf(c3 ? k3 : k4, V, c3 ? a3 : a4), 0.9f)),
+        float s = fmaf(c3 ? t3 : t4, UnitRoot::eval(__saturatef(fmaf(c3 ? k3 : k4, V, c3 ? a3 : a4))),
                        c3 ? b3 : 0.0f);
         if (V < V2) s = h2 - Fm<float>::sqrt_(fmaxf(fmaf(k2a, V, -k2b), 1e-30f));
         if (V < V1) s = fmaf(-cb1, Fm<float>::cbrt_(V), 0.5f);

@@ -26,7 +26,7 @@ __device__ __forceinline__ p2::f2 offset_two<M_SZ_OPT>(const CellPlic<M_SZ_OPT>&
     // the root of cases (3)/(4), as UnitRoot::eval
     const b2 c3 = lt(V, mk(P.V3));
     f2 a = fma(sel(c3, mk(P.k3), mk(P.k4)), V, sel(c3, mk(P.a3), mk(P.a4)));
-    a = make_float2(fminf(a.x, 0.9f), fminf(a.y, 0.9f));
+    a = make_float2(__saturatef(a.x), __saturatef(a.y));
     const f2 z = mul(a, a);
     f2 n = fma(mk(R::c4), z, mk(R::c3));
     n = fma(n, z, mk(R::c2));
