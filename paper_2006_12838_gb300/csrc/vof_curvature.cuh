@@ -296,23 +296,31 @@ struct CellPlic {
     }
 };
 
-// Root of u^3 - 3 u + 2 a = 0 on 0 <= a <= 0.886, divided by 2/3: the
-// trigonometric root 2 sin(asin(a)/3) of cases (3)/(4) in units of t (Q = 3 t^2;
-// see p2::centre_distance).  The odd polynomial of p2::depressed_root (there with
-// powers of 3^(1/2) folded in), negated, then one Newton step, u <- (2/3) (a -
-// u^3)/(1 - u^2), as a correction of 3/2 u: the reciprocal's error scales with the
-// correction alone (kappa of 24 small fields 2.91e-7 -> 2.89e-7 against 64 bits, the
-// arcsine form 2.92e-7; no difference in time).
-struct UnitRoot {
-    static constexpr float c0 = -0.6675798892974854f, c1 = -0.07909464836120605f,
-                           c2 = -0.1595292091369629f, c3 = 0.23291343450546265f,
-                           c4 = -0.2261897623538971f;
-    static __device__ __forceinline__ float eval(float a) {
-        const float z = a * a;
-        const float n = a * fmaf(fmaf(fmaf(fmaf(c4, z, c3), z, c2), z, c1), z, c0);   // -u
-        const float v = n * n;
-        const float m = -0.5f * n;
-        return fmaf(fmaf(m, v, fmaf(1.5f, n, a)), rcp_approx(1.0f - v), 3.0f * m);
+// The smaller positive root w of the depressed cubic w^3 - Q w + R = 0 of cases
+// (3)/(4) (p2::centre_distance) as a function of X = R/Q, its limit for small w: with
+// z = X^2/Q <= 0.1158 in these cases, w = X P(z) by the polynomial of
+// p2::depressed_root (signs turned), h = w^2/Q, and one Newton step on
+// w h - w + X = 0, w + (w h - w + X)/(1 - 3 h).  X is linear in the volume, k V + c, and
+// the step's residual takes c - w first, so that neither X's rounding nor the step's
+// stays in w; the constants of the normal are k, c and 1/Q.
+// |d0| error, rms, against 64 bits for random (nearly equal) components: case (3)
+// 2.1e-8 (2.4e-8), case (4) 1.2e-8 (1.8e-8); with the argument and the root in units of
+// (Q/3)^(1/2), five constants rounded before the volume is known, 3.3e-8 (7.3e-8) and
+// 1.4e-8 (2.7e-8); the arcsine and a Newton step on Eq. 10 2.6e-8 (2.5e-8) and
+// 2.9e-8 (2.7e-8).
+struct CentreRoot {
+    static constexpr float c0 = 1.001369833946228f, c1 = 0.8008332848548889f, c2 = 10.902824401855469f,
+                           c3 = -107.44769287109375f, c4 = 704.3350219726562f;
+    // z is held below 0.12: where m1 < 1e-14 m2 the thresholds' rounding lets volumes of
+    // cases (2) and (5) in, with X of either sign below 1e-7 and Q far below X^2
+    // (1/Q up to infinity: X^2/Q infinite or NaN, taken as 0.12).
+    static constexpr float zmax = 0.12f;
+    static __device__ __forceinline__ float eval(float k, float V, float c, float iq, float b) {
+        const float X = fmaf(k, V, c), z = fminf(X * X * iq, zmax);
+        const float p = fmaf(fmaf(fmaf(fmaf(c4, z, c3), z, c2), z, c1), z, c0);
+        const float w = X * p, h = p * p * z;
+        const float f = fmaf(w, h, fmaf(k, V, c - w));
+        return fmaf(f, rcp_approx(fmaf(-3.0f, h, 1.0f)), w + b);
     }
 };
 
@@ -321,18 +329,14 @@ struct UnitRoot {
 // cell use the centre normal, Eq. 36).  Per solve there remain: the reduced
 // volume, four threshold tests on V, the closed forms of cases (5), (2), (1)
 // (the last as cbrt(6 m1 m2 m3) * cbrt(V)), and the root of the depressed cubic
-// of cases (3)/(4) in units of t, whose argument a is linear in V: k3 V + a3 or
-// k4 V + a4 (p2::centre_distance).  Where m1 < 1e-14 m2 the thresholds' rounding lets
-// volumes of cases (2) and (5) in, for which a is the difference of two large numbers,
-// of either sign; t is then below 1e-7, and any a in [0, 1] (saturated) gives their
-// offset to rounding.  All as distances s = 1/2 - d from the
+// of cases (3)/(4) (CentreRoot).  All as distances s = 1/2 - d from the
 // cell's centre.  The thresholds are the product-form tests of
 // solve_sz_opt_default divided through once.
 template <>
 struct CellPlic<M_SZ_OPT> {
     float L, m3;
     float V5, V1, V2, V3;
-    float k3, a3, t3, b3, k4, a4, t4, k2a, k2b, h2, cb1;
+    float c3, i3, b3, k4, c4, i4, k2a, k2b, h2, cb1;
     __device__ __forceinline__ void prepare(float nx, float ny, float nz) {
         const float ax = fabsf(nx), ay = fabsf(ny), az = fabsf(nz);
         L = ax + ay + az;
@@ -351,36 +355,30 @@ struct CellPlic<M_SZ_OPT> {
         V1 = sq1 * rk;                                           // case (1): V < V1
         V2 = (sq1 - 3.0f * m2 * (m1 - m2)) * rk;                 // case (2): V < V2
         const float num3 = m3 * m3 * (3.0f * n12 - m3) + sq1 * (m1 - 3.0f * m3) + m2 * m2 * (m2 - 3.0f * m3);
-        V3 = (m3 < n12 && m1m2 > 0.0f) ? num3 * rk * inv1 : 3.4e38f;  // case (3): V < V3
-        // case (3): t^2 = 2 m1 m2, a = 3/4 (m1 + m2 - 2 m3 V) / t
-        const float t32 = 2.0f * m1m2;
-        const float r3 = recip_sqrt(t32);
-        t3 = t32 * r3 * (2.0f / 3.0f);
-        a3 = 0.75f * n12 * r3;
-        k3 = -1.5f * m3 * r3;
+        // (below 1e-30 case (4) is no wider than a rounding, and its constants overflow)
+        V3 = (m3 < n12 && m1m2 > 1e-30f) ? num3 * rk * inv1 : 3.4e38f;  // case (3): V < V3
+        // case (3): X = (m1 + m2)/2 - m3 V, Q = 6 m1 m2, s = 1/2 - m1 - m2 + w
+        c3 = 0.5f * n12;
+        i3 = rcp_approx(6.0f * m1m2);
         b3 = 0.5f - n12;
-        // case (4): t^2 = (m1 (2 (m2 + m3) - m1) - (m3 - m2)^2)/4, a = 3/4 m1 m2 m3 (1 - 2 V) / t^3
-        const float d32 = m3 - m2;
-        const float t42 = 0.25f * (m1 * (2.0f * (m2 + m3) - m1) - d32 * d32);
-        const float r4 = recip_sqrt(t42);
-        t4 = t42 * r4 * (2.0f / 3.0f);
-        a4 = 0.75f * m1m2 * m3 * r4 * r4 * r4;
-        k4 = -2.0f * a4;
+        // case (4): X = c (1 - 2 V), Q = 3/4 q, s = w with q = m1 (2 - 3 m1) - (m3 - m2)^2 and
+        // c = 2 m1 m2 m3 / q, a division with the products' roundings carried along
+        const float d32 = m3 - m2, e = fmaf(-3.0f, m1, 2.0f), me = m1 * e, q = fmaf(-d32, d32, me);
+        const float num = m1m2 * (2.0f * m3);
+        const float rnum = fmaf(m1m2, 2.0f * m3, -num) + 2.0f * m3 * fmaf(m1, m2, -m1m2);
+        const float r = rcp_approx(q), c = num * r;
+        c4 = fmaf(fmaf(-c, q, num) + fmaf(-c, fmaf(m1, e, -me), rnum), r, c);
+        k4 = -2.0f * c4;
+        i4 = (4.0f / 3.0f) * r;
         k2a = 2.0f * m2 * m3;
         k2b = sq1 * (1.0f / 12.0f);
         h2 = 0.5f - 0.5f * m1;
         cb1 = Fm<float>::cbrt_(k23 * m1);
     }
-    // 1/sqrt(x), 0 for x <= 0, with a Newton step (t and a carry its error)
-    static __device__ __forceinline__ float recip_sqrt(float x) {
-        const float r = x > 0.0f ? rsqrtf(x) : 0.0f;
-        return r * fmaf(-0.5f * x * r, r, 1.5f);
-    }
     __device__ __forceinline__ float offset(float V0) const {
         const float V = fminf(V0, 1.0f - V0);
-        const bool c3 = V < V3;
-        float s = fmaf(c3 ? t3 : t4, UnitRoot::eval(__saturatef(fmaf(c3 ? k3 : k4, V, c3 ? a3 : a4))),
-                       c3 ? b3 : 0.0f);
+        const bool three = V < V3;
+        float s = CentreRoot::eval(three ? -m3 : k4, V, three ? c3 : c4, three ? i3 : i4, three ? b3 : 0.0f);
         if (V < V2) s = h2 - Fm<float>::sqrt_(fmaxf(fmaf(k2a, V, -k2b), 1e-30f));
         if (V < V1) s = fmaf(-cb1, Fm<float>::cbrt_(V), 0.5f);
         if (V >= V5) s = m3 * (0.5f - V);

@@ -21,27 +21,27 @@ __device__ __forceinline__ p2::f2 offset_two(const CellPlic<METHOD>& pl, p2::f2 
 template <>
 __device__ __forceinline__ p2::f2 offset_two<M_SZ_OPT>(const CellPlic<M_SZ_OPT>& P, p2::f2 V0) {
     using namespace p2;
-    typedef UnitRoot R;
+    typedef CentreRoot R;
     const f2 V = make_float2(fminf(V0.x, 1.0f - V0.x), fminf(V0.y, 1.0f - V0.y));
-    // the root of cases (3)/(4), as UnitRoot::eval
-    const b2 c3 = lt(V, mk(P.V3));
-    f2 a = fma(sel(c3, mk(P.k3), mk(P.k4)), V, sel(c3, mk(P.a3), mk(P.a4)));
-    a = make_float2(__saturatef(a.x), __saturatef(a.y));
-    const f2 z = mul(a, a);
-    f2 n = fma(mk(R::c4), z, mk(R::c3));
-    n = fma(n, z, mk(R::c2));
-    n = fma(n, z, mk(R::c1));
-    n = mul(a, fma(n, z, mk(R::c0)));
-    const f2 v = mul(n, n);
-    const f2 m = mul(mk(-0.5f), n);
-    const f2 u = fma(fma(m, v, fma(mk(1.5f), n, a)), rcp(sub(mk(1.0f), v)), mul(mk(3.0f), m));
-    f2 s = fma(sel(c3, mk(P.t3), mk(P.t4)), u, sel(c3, mk(P.b3), mk(0.0f)));
+    // the root of cases (3)/(4), as CentreRoot::eval
+    const b2 three = lt(V, mk(P.V3));
+    const f2 k = sel(three, mk(-P.m3), mk(P.k4)), c = sel(three, mk(P.c3), mk(P.c4));
+    const f2 X = fma(k, V, c);
+    f2 z = mul(mul(X, X), sel(three, mk(P.i3), mk(P.i4)));
+    z = make_float2(fminf(z.x, R::zmax), fminf(z.y, R::zmax));
+    f2 p = fma(mk(R::c4), z, mk(R::c3));
+    p = fma(p, z, mk(R::c2));
+    p = fma(p, z, mk(R::c1));
+    p = fma(p, z, mk(R::c0));
+    const f2 w = mul(X, p), h = mul(mul(p, p), z);
+    const f2 f = fma(w, h, fma(k, V, sub(c, w)));
+    f2 s = fma(f, rcp(fma(mk(-3.0f), h, mk(1.0f))), add(w, sel(three, mk(P.b3), mk(0.0f))));
     // cases (2), (1), (5)
     s = sel(lt(V, mk(P.V2)), sub(mk(P.h2), sqrtp(fmax0(fma(mk(P.k2a), V, mk(-P.k2b))))), s);
     s = sel(lt(V, mk(P.V1)), fma(mk(-P.cb1), cbrt_(V), mk(0.5f)), s);
     s = sel(le(mk(P.V5), V), mul(mk(P.m3), sub(mk(0.5f), V)), s);
-    const f2 h = mul(mk(P.L), s);
-    return make_float2(copysignf(h.x, V0.x - 0.5f), copysignf(h.y, V0.y - 0.5f));
+    s = mul(mk(P.L), s);
+    return make_float2(copysignf(s.x, V0.x - 0.5f), copysignf(s.y, V0.y - 0.5f));
 }
 
 }  // namespace plic
