@@ -192,7 +192,9 @@ FX_D bool root_cubic(const Task& c, u64& s) {
     const int e1 = exponent(c.b1), e2 = exponent(c.b2), ea = exponent(c.a);
     const u64 M1 = mantissa(c.b1), M2 = mantissa(c.b2);
     const i64 yh = (i64)(fixed(c.y & ABS) >> 1), Y = c.y >> 63 ? -yh : yh;       // y/2
-    const u64 N1 = shr(M1, 2 - e1), N2 = shr(M2, 2 - e2), N3 = N1 + N2 + (u64)(2 * Y);  // (case 4)
+    // (case 4)
+    const u64 N1 = shr(M1, 2 - e1), N2 = shr(M2, 2 - e2), N3 = N1 + N2 + (u64)(2 * Y);
+    const u64 D = N3 > N2 ? N3 - N2 : N2 - N3;
     float w;
     if (c1) {
         w = cbrt_start(6.0f * f1 * (f2 * (fa * 2.81474976710656e14f))) * 1.52587890625e-5f;  // 2^48, 2^-16
@@ -200,7 +202,10 @@ FX_D bool root_cubic(const Task& c, u64& s) {
         const float p3 = 3.0f * f1 * f2;
         float Q = 2.0f * p3;
         if (c4) {
-            const float f3 = (float)(uint32_t)(N3 >> 32) * 9.31322574615478515625e-10f, d = f3 - f2;  // 2^-30
+            // d = n3 - n2 < n1 from the exact difference, truncated (of two rounded floats it
+            // would leave Q < 0 where n1 < 1e-14)
+            const float f3 = (float)(uint32_t)(N3 >> 32) * 9.31322574615478515625e-10f;      // 2^-30
+            const float d = (float)(uint32_t)(D >> 32) * 9.31322574615478515625e-10f;
             Q = 0.75f * fmaf(f1, fmaf(2.0f, f2 + f3, -f1), -d * d);
         }
         const float rq = rsq(Q), x = (p3 * rq) * (fa * rq) * rq, z = x * x;
@@ -223,7 +228,6 @@ FX_D bool root_cubic(const Task& c, u64& s) {
     const u64 X = q3(mulhi(P12, c1 ? ((c.a << 11) | TOP) : fixed(c.a)));
     u64 q = c1 ? 0ull : P12 >> 1;
     if (c4) {
-        const u64 D = N3 > N2 ? N3 - N2 : N2 - N3;
         q = shr(mulhi(M1, ((N2 + N3) << 1) - N1), 2 + e2) - shl(mulhi(D, shl(D, -e1)), -e2);
     }
     const u64 R = c1 ? 0ull - shr(X, 1 + 2 * j - (e1 + e2 + ea)) : X;
