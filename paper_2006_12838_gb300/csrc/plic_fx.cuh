@@ -17,10 +17,12 @@
 // methods 1.1e-14.  With the set-up in fixed point as well the error was 5.9e-17, but
 // the kernel 359 instead of 285 us.
 //
-// Cells outside the scheme's range (a normal far from unit length, 0 < V0 or
-// 1 - V0 below 2^-96, invalid input) and those whose steps do not come out as
-// small as they must (none met in those 10^7) are refused, and the caller solves
-// them in FP64.  Nothing here needs the GPU: with FX_HOST defined and the few
+// The scheme takes normals with n3 in [1/2, 1 + 2^-20) and n1 < 3/4 as they are (all of
+// unit length; nothing in it assumes that), others times a power of two (rescale): the
+// offset is homogeneous in the normal, and the errors above then scale with it.
+// Cells with 0 < V0 or 1 - V0 below 2^-96, with L > 3 or n3 below 2^-60, invalid input and
+// those whose steps do not come out as small as they must (none met in those 10^7) are
+// refused, and the caller solves them in FP64.  Nothing here needs the GPU: with FX_HOST defined and the few
 // primitives below supplied, the functions compile for the host.
 #pragma once
 #include <stdint.h>
@@ -72,13 +74,40 @@ FX_D void sort(u64& b1, u64& b2, u64& b3) {
     t = c ? b2 : b1; b2 = c ? b1 : b2; b1 = t;
 }
 
-// Whether the scheme takes the cell (sorted |n|, V0's bits): n3 in [1/2, 1 +
+// Whether the scheme takes the cell as it is (sorted |n|, V0's bits): n3 in [1/2, 1 +
 // 2^-20) and n1 < 3/4 (then L < 3), and V0 = 0, in [2^-96, 1) or 1.
-FX_D bool in_range(u64 b1, u64 b3, u64 v0) {
-    const uint32_t h1 = (uint32_t)(b1 >> 32), h3 = (uint32_t)(b3 >> 32), hv = (uint32_t)(v0 >> 32);
-    return h3 - 0x3fe00000u <= 0x00100000u && h1 < 0x3fe80000u &&
-           (hv - (927u << 20) < 0x3ff00000u - (927u << 20) || (v0 & ABS) == 0ull || v0 == ONE);
+FX_D bool volume_in_range(u64 v0) {
+    const uint32_t hv = (uint32_t)(v0 >> 32);
+    return hv - (927u << 20) < 0x3ff00000u - (927u << 20) || (v0 & ABS) == 0ull || v0 == ONE;
 }
+FX_D bool in_range(u64 b1, u64 b3, u64 v0) {
+    const uint32_t h1 = (uint32_t)(b1 >> 32), h3 = (uint32_t)(b3 >> 32);
+    return h3 - 0x3fe00000u <= 0x00100000u && h1 < 0x3fe80000u && volume_in_range(v0);
+}
+
+// b 2^k for the bits of a non-negative double (0 below the normal range).
+FX_D u64 times2(u64 b, int k) {
+    const int e = (int)(b >> 52);
+    return e > 0 && e + k > 0 ? b + ((u64)(i64)k << 52) : 0ull;
+}
+
+// A normal outside the range brought into it by a power of two, exactly: n3 to [1/2,
+// 1), halved once more where n1 then is 3/4 or more (L up to 3) or n2 31/32 or more (case
+// (2) with w near 1).  k: its exponent (|k| < 64), by which d0 is to be divided; false
+// where L > 3 (a little less: the closed forms decide) or n3 < 2^-60.
+FX_D bool rescale(u64& b1, u64& b2, u64& b3, int& k) {
+    const uint32_t h3 = (uint32_t)(b3 >> 32);
+    if (h3 - (963u << 20) >= (62u << 20)) return false;
+    k = 1022 - (int)(h3 >> 20);
+    if (k < 0 && asd(b1) + asd(b2) + asd(b3) > 2.99999999) return false;
+    k -= (uint32_t)(times2(b1, k) >> 32) >= 0x3fe80000u || (uint32_t)(times2(b2, k) >> 32) >= 0x3fef0000u;
+    b1 = times2(b1, k);
+    b2 = times2(b2, k);
+    b3 = times2(b3, k);
+    return true;
+}
+// d0 of the cell itself, from that of the scaled one (bits, any sign).
+FX_D u64 unscale(u64 d0, int k) { return (d0 & ABS) == 0ull ? d0 : d0 - ((u64)(i64)k << 52); }
 
 // A non-negative double's bits as M 2^(e - 64) with the leading bit of M set (M =
 // 0 below 2^-61), and in units of 2^-62 (truncated).
@@ -184,11 +213,10 @@ FX_D bool root_square(const Task& c, u64& s) {
 
 // Cases (3), (4): w^3 - Q w + R = 0 (p2::centre_distance); case (1): w^3 =
 // 6 n1 n2 n3 V.  The residual 4 w^3 - 4 Q w + 4 R scaled by 2^-(e1 + e2), or
-// 4 w^3 - 24 n1 n2 n3 V by 2^-2j.
-template <int CODE>
-FX_D bool root_cubic(const Task& c, u64& s) {
+// 4 w^3 - 24 n1 n2 n3 V by 2^-2j.  c1, c4: case (1), (4); with them known at compile time the
+// selections fold away.
+FX_D bool root_cubic(const Task& c, bool c1, bool c4, u64& s) {
     const float f1 = flt(c.b1), f2 = flt(c.b2), fa = flt(c.a);
-    constexpr bool c1 = CODE == 1, c4 = CODE == 4;
     const int e1 = exponent(c.b1), e2 = exponent(c.b2), ea = exponent(c.a);
     const u64 M1 = mantissa(c.b1), M2 = mantissa(c.b2);
     const i64 yh = (i64)(fixed(c.y & ABS) >> 1), Y = c.y >> 63 ? -yh : yh;       // y/2
@@ -255,16 +283,16 @@ FX_D bool offset(u64 nx, u64 ny, u64 nz, u64 v0, u64& d0) {
     u64 b1 = nx & ABS, b2 = ny & ABS, b3 = nz & ABS, s;
     const u64 va = v0 & ABS;
     sort(b1, b2, b3);
-    if (!in_range(b1, b3, v0)) return false;
+    int k = 0;
+    if (!in_range(b1, b3, v0) && !(volume_in_range(v0) && rescale(b1, b2, b3, k))) return false;
     Task t;
     const int code = classify(b1, b2, b3, va, t, s);
     if (code == 5) {
-        d0 = va < HALF ? s | TOP : s;
+        d0 = unscale(va < HALF ? s | TOP : s, k);
         return true;
     }
-    const bool ok = code == 2 ? root_square(t, s) : code == 3 ? root_cubic<3>(t, s)
-                  : code == 4 ? root_cubic<4>(t, s) : root_cubic<1>(t, s);
-    d0 = round_s(s, va < HALF);
+    const bool ok = code == 2 ? root_square(t, s) : root_cubic(t, code == 1, code == 4, s);
+    d0 = unscale(round_s(s, va < HALF), k);
     return ok;
 }
 

@@ -355,22 +355,31 @@ k_plic_offset_pair(const float* __restrict__ nx, const float* __restrict__ ny,
 }
 
 // The optimised SZ and the analytic solution in PLIC_FP64 and
-// PLIC_FP64_REFINED: the scheme of plic_fx.cuh, and the closed forms in FP64 for the
-// cells it refuses (a call, to keep their registers out of the loop).
+// PLIC_FP64_REFINED: the scheme of plic_fx.cuh, and for the cells that the kernel below
+// leaves over the same scheme on the rescaled normal, one thread per cell, or the closed
+// forms in FP64 (a call, to keep their registers out of the loop).  2^24 cells: normals of
+// unit L1 length 452 us, of length 0.3 630 and 1.2 583 (all or half of the cells outside the
+// range; by the closed forms, called as the cells were read, 4880, 4820 and 4190; packed
+// closed forms 3165, double-float steps 585).  The rescaled cells packed by case as well
+// came to 450, 440 and 510, but the unaligned arrays' loop then to 194 us per 10 M cells of
+// unit normals, against 184.
 template <int METHOD>
-__device__ __noinline__ double offset_cell_slow(double nx, double ny, double nz, double V0, int* bad) {
+__device__ __noinline__ fx::u64 fx_rest(double nx, double ny, double nz, double V0, int& bad) {
+    fx::u64 d0;
+    if (fx::offset(fx::bits(nx), fx::bits(ny), fx::bits(nz), fx::bits(V0), d0)) return d0;
     int b = 0;
-    const double r = offset_cell<METHOD, double, false, false>(nx, ny, nz, V0, b);
-    *bad += b;
-    return r;
+    d0 = fx::bits(offset_cell<METHOD, double, false, false>(nx, ny, nz, V0, b));
+    bad += b;
+    return d0;
 }
 
 // Both methods and precisions are this kernel.  The cases are packed: FX_CELLS cells
-// per block and trip; every thread reads its four cells and settles case (5) and the
-// refused ones; the others leave their task in shared memory and their place in the
-// list of their case (lanes of one case share a counter's increment; the order in a
-// list does not matter); the warps take 32 cells of one list at a time; every thread
-// stores its own cells.  The arrays are read as integers: of the bits of a double in
+// per block and trip; every thread reads its four cells and settles case (5); the others
+// leave their task in shared memory and their place in the
+// list of their case, or in list 0 where the scheme does not take them as they are (lanes
+// of one list share a counter's increment; the order in a
+// list does not matter); the warps take 32 cells of one list at a time, list 0 last;
+// every thread stores its own cells.  The arrays are read as integers: of the bits of a double in
 // a register the compiler makes |x| an operation on the FP64 pipe (three per cell:
 // 396 against 317 us).
 // Bound: instruction issue (477 warp instructions per 32 cells, 72 % of the slots; ALU
@@ -393,14 +402,14 @@ k_plic_offset_fx(const double* __restrict__ nx, const double* __restrict__ ny,
     typedef fx::i64 i64;
     // a cell's task: b1 (with V0 < 1/2 in its sign), b2 and a, y; its d0 then in hi.y
     __shared__ ulonglong2 lo[FX_CELLS], hi[FX_CELLS];
-    __shared__ unsigned short list[4][FX_CELLS];        // the cells of cases (1) to (4)
-    __shared__ int count[4];
+    __shared__ unsigned short list[5][FX_CELLS];        // the cells of cases (1) to (4); 0: the others
+    __shared__ int count[5];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int bad = 0;
     for (int64_t i0 = (int64_t)blockIdx.x * FX_CELLS; i0 < n; i0 += (int64_t)gridDim.x * FX_CELLS) {
         const int cells = (int)(n - i0 < FX_CELLS ? n - i0 : FX_CELLS);
         const bool vec = VEC && cells == FX_CELLS;
-        if (threadIdx.x < 4) count[threadIdx.x] = 0;
+        if (threadIdx.x < 5) count[threadIdx.x] = 0;
         __syncthreads();
         auto place = [&](int j) { return vec ? 2 * (FX_THREADS * (j >> 1) + (int)threadIdx.x) + (j & 1)
                                              : FX_THREADS * j + (int)threadIdx.x; };
@@ -409,10 +418,11 @@ k_plic_offset_fx(const double* __restrict__ nx, const double* __restrict__ ny,
             if (i < cells) {
                 u64 b1 = ax & fx::ABS, b2 = ay & fx::ABS, b3 = az & fx::ABS;
                 const u64 va = v & fx::ABS, sign = va < fx::HALF ? fx::TOP : 0ull;
-                u64 s;
                 fx::sort(b1, b2, b3);
+                code = 0;
                 if (fx::in_range(b1, b3, v)) {
                     fx::Task t;
+                    u64 s;
                     code = fx::classify(b1, b2, b3, va, t, s);
                     if (code != 5) {
                         lo[i] = make_ulonglong2(t.b1 | sign, t.b2);
@@ -421,17 +431,15 @@ k_plic_offset_fx(const double* __restrict__ nx, const double* __restrict__ ny,
                     } else {
                         s |= sign;
                     }
-                } else {
-                    s = fx::bits(offset_cell_slow<METHOD>(fx::asd(ax), fx::asd(ay), fx::asd(az), fx::asd(v), &bad));
+                    hi[i].y = s;
                 }
-                hi[i].y = s;
             }
             const unsigned same = __match_any_sync(0xffffffffu, code);
             const int first = __ffs(same) - 1;
             int at = 0;
-            if (lane == first && code != 5) at = atomicAdd(&count[code - 1], __popc(same));
+            if (lane == first && code != 5) at = atomicAdd(&count[code], __popc(same));
             at = __shfl_sync(0xffffffffu, at, first) + __popc(same & ((1u << lane) - 1u));
-            if (code != 5) list[code - 1][at] = (unsigned short)i;
+            if (code != 5) list[code][at] = (unsigned short)i;
         };
         if (vec) {
 #pragma unroll 1
@@ -455,27 +463,36 @@ k_plic_offset_fx(const double* __restrict__ nx, const double* __restrict__ ny,
         }
         __syncthreads();
         // 32 cells of a case at a time, the longest roots first
-        const int c1 = count[0], c2 = count[1], c3 = count[2], c4 = count[3];
+        const int c1 = count[1], c2 = count[2], c3 = count[3], c4 = count[4];
         const int t4 = (c4 + 31) >> 5, t3 = t4 + ((c3 + 31) >> 5), t1 = t3 + ((c1 + 31) >> 5),
                   t2 = t1 + ((c2 + 31) >> 5);
         for (int t = warp; t < t2; t += FX_THREADS / 32) {
             const int code = t < t4 ? 4 : t < t3 ? 3 : t < t1 ? 1 : 2;
             const int k = 32 * (t - (t < t4 ? 0 : t < t3 ? t4 : t < t1 ? t3 : t1)) + lane;
             if (k < (code == 4 ? c4 : code == 3 ? c3 : code == 1 ? c1 : c2)) {
-                const int i = list[code - 1][k];
+                const int i = list[code][k];
                 const ulonglong2 p = lo[i], q = hi[i];
                 const fx::Task c = {p.x & fx::ABS, p.y, q.x, q.y};
                 u64 s;
                 bool ok;
                 if (code == 2) ok = fx::root_square(c, s);
-                else if (code == 3) ok = fx::root_cubic<3>(c, s);
-                else if (code == 4) ok = fx::root_cubic<4>(c, s);
-                else ok = fx::root_cubic<1>(c, s);
-                hi[i].y = ok ? fx::round_s(s, (i64)p.x < 0)
-                             : fx::bits(offset_cell_slow<METHOD>(nx[i0 + i], ny[i0 + i], nz[i0 + i], V0[i0 + i], &bad));
+                else if (code == 3) ok = fx::root_cubic(c, false, false, s);
+                else if (code == 4) ok = fx::root_cubic(c, false, true, s);
+                else ok = fx::root_cubic(c, true, false, s);
+                hi[i].y = fx::round_s(s, (i64)p.x < 0);
+                if (!ok) list[0][atomicAdd(&count[0], 1)] = (unsigned short)i;
             }
         }
         __syncthreads();
+        const int rest = count[0];
+        if (rest > 0) {
+            for (int k = threadIdx.x; k < rest; k += FX_THREADS) {
+                const int i = list[0][k];
+                const int64_t q = i0 + i;
+                hi[i].y = fx_rest<METHOD>(nx[q], ny[q], nz[q], V0[q], bad);
+            }
+            __syncthreads();
+        }
         if (vec) {
 #pragma unroll
             for (int k = 0; k < 2; ++k)

@@ -24,8 +24,33 @@ int main(int argc, char** argv) {
             n[2] = n[1] * (1 + (u(r) < 0.5 ? (int)(4 * u(r)) * 1.2e-16 : 2 * e * u(r)));
             v = 0.5 + (u(r) < 0.5 ? -1 : 1) * std::pow(10, -12 - 5 * u(r));
         }
+        if (kind > 0) {
+            // off unit length: 1/2 to 2; unit L1 length; down to 2^-58; components near 3/4
+            double scale = 1, l = 0;
+            for (double& x : n) x = g(r);
+            if (u(r) < 0.3) n[0] *= std::pow(10, -17 * u(r));
+            if (u(r) < 0.3) n[1] = n[0] * (1 + std::pow(10, -16 * u(r)));
+            if (u(r) < 0.3) n[2] = n[1] * (1 + std::pow(10, -16 * u(r)));
+            for (double x : n) l += kind == 2 ? std::fabs(x) : x * x;
+            if (kind != 2) l = std::sqrt(l);
+            if (kind == 1) scale = std::pow(2, 2 * u(r) - 1);
+            if (kind == 3) scale = std::pow(2, -58 * u(r));
+            if (kind == 4) scale = 0.75 + 0.25 * u(r);
+            const bool near = kind == 4 && u(r) < 0.5;
+            for (double& x : n) x = near ? 0.374 + 0.63 * u(r) : x * scale / l;
+        }
         for (int k = 0; k < 3; ++k) a[k] = n[k];
         order(a);
+        if (a[0] + a[1] + a[2] > 2.999 || a[2] < std::pow(2, -59.9)) continue;
+        if (kind > 0 && u(r) < 0.4) {                    // at and beside the case boundaries
+            const quad half = ((quad)a[0] + a[1] + a[2]) / 2;
+            const quad at[5] = {a[0], a[1], a[2], (quad)a[0] + a[1], half};
+            quad d = at[(int)(5 * u(r))] + std::pow(10, -17 * u(r)) * (u(r) < 0.5 ? -a[0] : a[0]);
+            d = d < 0 ? 0 : d > half ? half : d;
+            v = std::fmin((double)volume(d, a[0], a[1], a[2]), 0.5);
+            v = std::fmax(v, std::pow(2, -96));
+            if (u(r) < 0.5) v = 1 - v;
+        }
         u64 b[4], o;
         for (int k = 0; k < 3; ++k) memcpy(&b[k], &n[k], 8);
         memcpy(&b[3], &v, 8);

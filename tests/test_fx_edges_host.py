@@ -30,3 +30,14 @@ def test_sliver_beside_one_half(exe):
     of the 2e-16 of test_fx_host.py is half the rounding of n1 + n2 and of y/2."""
     refused, worst, shifts = _run(exe, 0)
     assert (refused, shifts) == (0, 0) and worst <= 2e-16, (refused, worst, shifts)
+
+
+@pytest.mark.parametrize("kind", [1, 2, 3, 4])
+def test_normals_off_unit_length(exe, kind):
+    """Lengths 1/2 to 2, unit L1 length, lengths down to 2^-58, components around 3/4: no
+    cell with L < 2.999 is refused, and of the power of two above n3 |d0 error| <= 4e-16:
+    half an ulp of s and of y/2 (below 1.5 and 1: 1.1e-16, 5.6e-17), half the rounding of
+    n1 + n2 (5.6e-17, all doubled where three components of 3/4 and more are halved once
+    more) and the root's own."""
+    refused, worst, shifts = _run(exe, kind)
+    assert (refused, shifts) == (0, 0) and worst <= 4e-16, (refused, worst, shifts)
