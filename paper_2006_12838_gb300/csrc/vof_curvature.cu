@@ -71,28 +71,51 @@ k_vof_curvature_batched(const vof_field* __restrict__ fields, const int64_t* __r
     }
 }
 
-// The batch's tables, passed by value: a kernel writes them to the workspace
-// (TABLE_FIELDS fields per launch, 3.6 KB of parameters) and clears the ticket;
-// the batch's kernel is launched behind it (pdl_wait).  Two copies from
+// The batch's tables, passed by value: a kernel writes them to the workspace and clears
+// the ticket; the batch's kernel is launched behind it (pdl_wait).  Two copies from
 // pageable memory and a memset in its place: 213.6 instead of 205 us per call of
 // the 64-field batch, and a captured call read the host's tables, long gone,
-// at each replay.
-constexpr int TABLE_FIELDS = 64;
+// at each replay.  Up to 64 fields go in one launch of 3.6 KB of parameters, more in
+// launches of 512 (28.7 KB; a launch takes at most 32 KB), a block of 64 threads per 64
+// fields.  Whole calls, lists of 607 cells (in brackets: launches of 64; the copies): 65
+// fields 12.4 us (14.7; 22.4), 300 21.0 (37.2; 30.0), 1000 52 (111; 61), 10 000 425 (982; 467).
+constexpr int TABLE_THREADS = 64;
+template <int N>
 struct BatchTable {
-    vof_field f[TABLE_FIELDS];
-    int64_t prefix[TABLE_FIELDS];        // list entries before each field
+    vof_field f[N];
+    int64_t prefix[N];                   // list entries before each field
     int first, count;
 };
 
-__global__ void k_batch_table(BatchTable t, vof_field* __restrict__ fields, int64_t* __restrict__ prefix,
-                              unsigned long long* __restrict__ ticket) {
-    const int i = threadIdx.x;
+template <int N>
+__global__ void __launch_bounds__(TABLE_THREADS)
+k_batch_table(const __grid_constant__ BatchTable<N> t, vof_field* __restrict__ fields, int64_t* __restrict__ prefix,
+              unsigned long long* __restrict__ ticket) {
+    const int i = blockIdx.x * TABLE_THREADS + threadIdx.x;
     if (i < t.count) {
         fields[t.first + i] = t.f[i];
         prefix[t.first + i] = t.prefix[i];
     }
     if (i == 0) *ticket = 0ull;
     pdl_trigger();
+}
+
+// Fields [first, first + count) of a batch, count <= N; `before`: the list entries before
+// them, moved on.
+template <int N>
+static cudaError_t launch_table(const vof_field* fields, size_t first, int count, int64_t& before, vof_field* d_fields,
+                                int64_t* d_pre, unsigned long long* d_ticket, cudaStream_t s) {
+    BatchTable<N> t;
+    t.first = (int)first;
+    t.count = count;
+    for (int j = 0; j < count; ++j) {
+        t.f[j] = fields[first + j];
+        t.prefix[j] = before;
+        before += t.f[j].n_iface;
+    }
+    void* args[] = {(void*)&t, (void*)&d_fields, (void*)&d_pre, (void*)&d_ticket};
+    return cudaLaunchKernel(reinterpret_cast<const void*>(&k_batch_table<N>),
+                            dim3((unsigned)((count + TABLE_THREADS - 1) / TABLE_THREADS)), dim3(TABLE_THREADS), args, 0, s);
 }
 
 #define PLIC_FIT_TABLE(K, M) \
@@ -236,18 +259,10 @@ extern "C" plic_status vof_curvature_batched(const vof_field* fields, int n_fiel
     cudaStream_t s = as_stream(stream);
     cudaError_t e = cudaSuccess;
     int64_t before = 0;
-    for (size_t i = 0; i < nf && e == cudaSuccess; i += TABLE_FIELDS) {
-        BatchTable t = {};
-        t.first = (int)i;
-        t.count = (int)(nf - i < TABLE_FIELDS ? nf - i : TABLE_FIELDS);
-        for (int j = 0; j < t.count; ++j) {
-            t.f[j] = fields[i + j];
-            t.prefix[j] = before;
-            before += t.f[j].n_iface;
-        }
-        void* targs[] = {(void*)&t, (void*)&d_fields, (void*)&d_pre, (void*)&d_ticket};
-        e = cudaLaunchKernel(reinterpret_cast<const void*>(&k_batch_table), dim3(1), dim3(TABLE_FIELDS), targs, 0, s);
-    }
+    for (size_t i = 0; i < nf && e == cudaSuccess; i += 512)
+        e = nf - i <= 64 ? launch_table<64>(fields, i, (int)(nf - i), before, d_fields, d_pre, d_ticket, s)
+                         : launch_table<512>(fields, i, (int)(nf - i < 512 ? nf - i : 512), before, d_fields, d_pre,
+                                             d_ticket, s);
     if (e != cudaSuccess) { set_last_error("vof_curvature_batched", e); return PLIC_ERR_CUDA; }
     const int64_t need = ((total + chunk - 1) / chunk + CO_WARPS - 1) / CO_WARPS;
     if (grid > need) grid = need;
