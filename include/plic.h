@@ -255,7 +255,8 @@ plic_status vof_laplace_pressure(const float *phi, int nx, int ny, int nz, const
  * respect to the fill field: g_phi = d(sum_k g_kappa[k] kappa[k]) / d phi,
  * with the interface set (idx and the neighbour flags 0 < phi < 1) held fixed.
  * g_phi is dense (nx*ny*nz floats) and overwritten (during the call it also
- * holds one mark per field cell).  Per interface cell the 27
+ * holds one mark per field cell); it may be phi itself, or overlap phi or g_kappa,
+ * whose values are then lost.  Per interface cell the 27
  * partial derivatives are written to the workspace and gathered per field
  * cell in a fixed order, so the result is deterministic (no floating-point
  * atomics).

@@ -23,7 +23,8 @@
 // deterministic, no floating-point atomics -- and writes 0 everywhere else.
 // Which cells j those are is marked in one bit per field cell; the marks live
 // in g_phi itself (the first words of each run of 1024 cells, read by the one
-// warp that then writes the run).  The map from a field cell to its list entry
+// warp that then writes the run; where g_phi overlaps an input, as in a gradient in
+// place, they are set by a kernel of their own once the reverse pass has read it).  The map from a field cell to its list entry
 // is not cleared: entry s of cell c counts only if idx[s] == c.
 // Only the foot-point variant (Eq. 36) is differentiated.
 //
@@ -70,6 +71,25 @@ k_curv_clear_marks(float* __restrict__ g_phi, int64_t cells) {
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words;
          w += (int64_t)gridDim.x * blockDim.x)
         *mark_word(g_phi, (unsigned)(32 * w)) = 0u;
+}
+
+// Marks the 27 cells of the stencil of cell c: three bits per row.
+__device__ __forceinline__ void mark_stencil(float* g_phi, int c, int nx, int nxy) {
+#pragma unroll
+    for (int r = 0; r < 9; ++r) {
+        const unsigned j = (unsigned)(c + (r % 3 - 1) * nx + (r / 3 - 1) * nxy - 1);
+        const unsigned sh = j & 31u;
+        atomicOr(mark_word(g_phi, j), 7u << sh);
+        if (sh > 29u) atomicOr(mark_word(g_phi, j + 2u), 7u >> (32u - sh));
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_curv_mark(const int32_t* __restrict__ idx, int64_t n, const int64_t* __restrict__ d_n, int nx, int nxy,
+            float* __restrict__ g_phi) {
+    const int64_t lim = d_n && *d_n < n ? *d_n : n;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < lim; k += (int64_t)gridDim.x * blockDim.x)
+        mark_stencil(g_phi, __ldg(idx + k), nx, nxy);
 }
 
 // Area and centroid of the cut polygons of a cell's planes (all with the
@@ -134,7 +154,8 @@ struct CellArea {
 // two neighbours per trip in the forward loop, whose offsets stay in the
 // entry's row of shared memory for the reverse loop, which leaves the entry's
 // partial derivatives there; the block then writes its rows out together.
-// The thread also marks its stencil in g_phi and enters itself into the map.
+// The thread also marks its stencil in g_phi (unless that is null) and enters itself into
+// the map.
 template <int METHOD, int FIT>
 __global__ void __launch_bounds__(CB_THREADS)
 k_vof_curvature_vjp(const float* __restrict__ phi, int nx, int ny, const int32_t* __restrict__ idx,
@@ -164,13 +185,7 @@ k_vof_curvature_vjp(const float* __restrict__ phi, int nx, int ny, const int32_t
         if (on) {
             slot[c] = (int32_t)k;
             phi0 = __ldg(p0);
-#pragma unroll
-            for (int r = 0; r < 9; ++r) {            // the 27 cells j: three bits per row
-                const unsigned j = (unsigned)(c + (r % 3 - 1) * nx + (r / 3 - 1) * nxy - 1);
-                const unsigned sh = j & 31u;
-                atomicOr(mark_word(g_phi, j), 7u << sh);
-                if (sh > 29u) atomicOr(mark_word(g_phi, j + 2u), 7u >> (32u - sh));
-            }
+            if (g_phi) mark_stencil(g_phi, c, nx, nxy);
             for_e27<1>([&](auto I) {
                 constexpr int i = decltype(I)::value;
                 constexpr int p = E27Table::v[i];
@@ -507,7 +522,15 @@ extern "C" plic_status vof_curvature_backward(const float* phi, int nx, int ny, 
         return check_launch("vof_curvature_backward");
     }
     const int cg = stride_grid(reinterpret_cast<const void*>(&k_curv_clear_marks), 256, (cells + 31) / 32);
-    k_curv_clear_marks<<<cg, 256, 0, s>>>(g_phi, cells);
+    // the reverse pass reads phi and g_kappa: marks in g_phi before or during it only where
+    // they lie elsewhere
+    auto inside = [&](const float* p, int64_t count) {
+        const uintptr_t a = (uintptr_t)p, g = (uintptr_t)g_phi;
+        return a < g + (uintptr_t)cells * sizeof(float) && g < a + (uintptr_t)count * sizeof(float);
+    };
+    const bool in_place = inside(phi, cells) || inside(g_kappa, n_iface);
+    float* marks = in_place ? nullptr : g_phi;
+    if (marks) k_curv_clear_marks<<<cg, 256, 0, s>>>(marks, cells);
     // the same fit policy as the forward call: adaptive unless a FIT flag is given
     const int fit = (flags & PLIC_FLAG_FIT_DF32) ? FIT_DF32 : (flags & PLIC_FLAG_FIT_FP32) ? FIT_FP32
                   : (flags & PLIC_FLAG_FIT_FP64) ? FIT_FP64 : FIT_AUTO;
@@ -521,10 +544,15 @@ extern "C" plic_status vof_curvature_backward(const float* phi, int nx, int ny, 
     }
     const int grid = stride_grid(k, CB_THREADS, n_iface);
     void* args[] = {(void*)&phi, (void*)&nx, (void*)&ny, (void*)&idx, (void*)&n_iface,
-                    (void*)&d_n_iface, (void*)&g_kappa, (void*)&contrib, (void*)&slot, (void*)&g_phi,
+                    (void*)&d_n_iface, (void*)&g_kappa, (void*)&contrib, (void*)&slot, (void*)&marks,
                     (void*)&flags};
     const cudaError_t e = cudaLaunchKernel(k, dim3(grid), dim3(CB_THREADS), args, 0, s);
     if (e != cudaSuccess) { set_last_error("vof_curvature_backward", e); return PLIC_ERR_CUDA; }
+    if (in_place) {
+        k_curv_clear_marks<<<cg, 256, 0, s>>>(g_phi, cells);
+        const int mg = stride_grid(reinterpret_cast<const void*>(&k_curv_mark), 256, n_iface);
+        k_curv_mark<<<mg, 256, 0, s>>>(idx, n_iface, d_n_iface, nx, nx * ny, g_phi);
+    }
     const int vec = aligned(g_phi, 16);
     const int gg = stream_grid(reinterpret_cast<const void*>(&k_curv_gather), 256, (cells + RUN - 1) / RUN * 256 / GATHER_RUNS + 255);
     k_curv_gather<<<gg, 256, 0, s>>>(idx, n_iface, d_n_iface, slot, contrib, nx, ny, cells, g_phi, vec);
