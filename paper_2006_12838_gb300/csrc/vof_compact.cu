@@ -38,37 +38,6 @@ namespace plic {
 
 constexpr int CT_THREADS = 256;
 constexpr int CT_WARPS = CT_THREADS / 32;
-// tiles or blocks of tiles whose counts the write pass sums in front of each block
-constexpr int64_t CT_MAX_SUPERS = 8192;
-
-// How a field is cut: cells [base, base + cells) of the flat field (base a
-// multiple of 32 cells), tiles of `tile` cells, S tiles per block of pass 1.
-struct CompactPlan {
-    int64_t base, cells, tiles, supers;
-    int tile, S;
-};
-
-// Tile sizes: 8192 cells (16 loads of 16 bytes per lane in flight) where that
-// fills the chip more than twice (2560 blocks and up), smaller tiles below, where
-// the last blocks and, smaller still, a single block set the time (64^3: 248 tiles
-// of 1024 cells 5.9 us, 32 tiles of 8192 14 us; with the curvature after it, 256^3
-// 24.0 us with 8192 cells and 23.6 with 4096, 301 x 203 x 257 24.0 and 23.7,
-// 1 GiB 215 and 219).  S grows once the write pass would have to sum more
-// than CT_MAX_SUPERS counts (above 67 M cells; one scan launch in between took
-// 11 us on 1 GiB).
-static CompactPlan compact_plan(int nx, int ny, int nz) {
-    CompactPlan p;
-    const int64_t nxy = (int64_t)nx * ny;
-    p.base = nxy & ~(int64_t)31;
-    p.cells = nxy * (nz - 1) - p.base;
-    p.tile = p.cells >= (int64_t)20 << 20 ? 8192 : p.cells >= (int64_t)1 << 20 ? 4096 : 1024;
-    p.tiles = (p.cells + p.tile - 1) / p.tile;
-    p.S = 1;
-    while ((p.tiles + p.S - 1) / p.S > CT_MAX_SUPERS) p.S *= 2;
-    p.supers = (p.tiles + p.S - 1) / p.S;
-    return p;
-}
-
 // The interface test 0 < phi < 1 on the float's bits: the positive floats
 // below 1.0f are exactly the bit patterns 1 .. 0x3F7FFFFF (zero, negative
 // values, 1.0f and above, infinities and NaNs all fall outside).
@@ -438,25 +407,12 @@ static cudaError_t compact_passes(const float* phi, int nx, int ny, int nz, cons
                             : launch_compact<false>(phi, g, p, info, bits, idx, cap, d_count, s);
 }
 
-// Ints of scratch before the bits: tile infos and block sums.
-static int64_t info_ints(const CompactPlan& p) {
-    return (p.tiles + 3) / 4 * 4 + (p.S > 1 ? p.supers : 0);
-}
-
 }  // namespace plic
 
 extern "C" size_t plic_workspace_bytes(int op, int64_t arg) {
     if (arg < 0) return 0;
     switch (op) {
-        case PLIC_WS_COMPACT: {
-            // two words per 8192 cells and one per 16 cells: room for the tile
-            // infos and block sums (at most one word per 819 cells) and the
-            // interface bits (one word per 32 cells) of any field of arg cells
-            const int64_t t = (arg + 8191) / 8192 * 2 + 1;
-            const size_t a = ((size_t)t * sizeof(int) + 255) / 256 * 256;
-            const size_t b = ((size_t)(arg / 16 + 1) * sizeof(unsigned) + 255) / 256 * 256;
-            return a + b;
-        }
+        case PLIC_WS_COMPACT: return plic::compact_workspace(arg);
         case PLIC_WS_BATCHED: return plic::batch_workspace((size_t)arg);
         default: return 0;
     }
@@ -482,14 +438,8 @@ extern "C" plic_status vof_interface_compact(const float* phi, int nx, int ny, i
     if (!aligned(phi, 4) || (idx && !aligned(idx, 4)) || !aligned(workspace, 256)) return PLIC_ERR_ALIGN;
     const CompactPlan p = compact_plan(nx, ny, nz);
     int* info = reinterpret_cast<int*>(workspace);
-    const size_t info_bytes = ((size_t)info_ints(p) * sizeof(int) + 255) / 256 * 256;
-    // whole chunks of bits (512 cells)
-    const size_t bits_bytes = (size_t)((p.cells + 511) / 512) * 64;
-    unsigned* bits = nullptr;
-    if (info_bytes + bits_bytes <= ws_bytes)
-        bits = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(workspace) + info_bytes);
-    else if (info_bytes > ws_bytes)
-        return PLIC_ERR_ARG;
+    if (compact_bytes(p) > ws_bytes) return PLIC_ERR_ARG;
+    unsigned* bits = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(workspace) + compact_bits(p));
     const cudaError_t e = compact_passes(phi, nx, ny, nz, p, info, bits, idx, idx_capacity, d_count, s);
     if (e != cudaSuccess) { set_last_error("vof_interface_compact", e); return PLIC_ERR_CUDA; }
     return check_launch("vof_interface_compact");

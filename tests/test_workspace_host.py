@@ -25,9 +25,13 @@ def test_batch_layout_inside_the_workspace(lines):
     assert lines[0] == 0, "%d counts of fields end beyond the workspace" % lines[0]
 
 
+def test_compaction_layout_inside_the_workspace(lines):
+    assert lines[1] == 0, "%d shapes" % lines[1]
+
+
 def test_batch_size_query(lines):
     B.build()
-    sizes = lines[1:]
+    sizes = lines[2:]
     assert [plic.workspace_bytes(plic.WS_BATCHED, n) for n in range(len(sizes))] == sizes
     # sizes that callers hold from before stay enough
     assert sizes == [(56 * n + 16 + 255) // 256 * 256 + 256 for n in range(len(sizes))]
