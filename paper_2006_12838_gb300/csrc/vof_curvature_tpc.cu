@@ -96,9 +96,10 @@ __device__ __forceinline__ float tpc_kappa(const float* __restrict__ phi, int nx
 #pragma unroll
     for (int q = 0; q < 20; ++q) rec[q] = 0.0f;
     rec[20] = (float)((int)(tail - sv) / TPC_THREADS);
-    *tail = make_float2(phi0, __int_as_float(0));
+    *tail = make_float2(0.5f, __int_as_float(0));
     // two neighbours per trip (in ascending order; an odd last one pairs with
-    // the centre, the zero point behind the list, which adds nothing)
+    // the zero point behind the list, which adds nothing: its fill is 1/2, not phi0,
+    // which the caller's list may have outside [0, 1], where the paired solve is NaN)
 #pragma unroll 1
     for (const float2* r = sv; r < tail; r += 2 * TPC_THREADS) {
         const float2 r1 = r[0], r2 = r[TPC_THREADS];
