@@ -205,7 +205,8 @@ k_vof_curvature_vjp(const float* __restrict__ phi, int nx, int ny, const int32_t
         const float gl = sqrtf(gx * gx + gy * gy + gz * gz);
         float gbx = 0.0f, gby = 0.0f, gbz = 0.0f;
         const int m = __popc(mask);
-        if (gl > 0.0f && gk != 0.0f && m > 0) {
+        // (a listed cell whose own fill is not finite has no gradient)
+        if (gl > 0.0f && gk != 0.0f && m > 0 && fabsf(phi0) <= 3.40282347e38f) {
             const float inv = -1.0f / gl;
             const float nx_ = gx * inv, ny_ = gy * inv, nz_ = gz * inv;
             // ---- frame: u = n x r, b_y = u/|u|, b_x = b_y x n (Sec. 4.2) ----
