@@ -167,7 +167,9 @@ class ClockSampler:
 #   case test 7, the coefficients 2 / 6, the root of the depressed cubic 17 +
 #   rsqrt + div (polynomial start and one Newton step) and 2 for the offset;
 # * the same two in FP64 and FP64_REFINED (plic_fx.cuh): 6 FP64 operations per cell;
-#   the rest runs on the integer and FP32 pipes, for which there is no probe;
+#   the rest runs on the integer and FP32 pipes, for which there is no probe, so the
+#   fraction reported is that of the FP64 pipe alone (the kernel is bound by
+#   instruction issue: "counted" says so beside it);
 # * Kawano's SZ: its thresholds (10 + 2 div; 16 + 2 div more where cases
 #   (3)-(5) are told apart), the closed forms, and for (3)/(4) Viete's root
 #   (12 + sqrt, div, acos, cos);
@@ -582,6 +584,8 @@ def section_fp64(dev, pk, steps, cells, hist=None, pp=None, samples=None):
                 if prec == "fp64" or m in CENTRE:
                     eq = fp64_equivalents(m, hist, pp["fp64_call_fma_equiv"])
                     r["roofline"] = op_roofline(spc, 40.0, pk, pp, fp64=eq)
+                    if m in CENTRE:
+                        r["roofline"]["counted"] = "bytes and FP64 operations; bound by issue, not counted"
                 else:
                     fp, mu = fp32_pipes(m, "fp32p", hist)
                     r["roofline"] = op_roofline(spc, 40.0, pk, pp, fp32=fp + REFINE_FP32, mufu=mu)

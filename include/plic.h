@@ -61,12 +61,17 @@ typedef enum {
 
 typedef enum {
     PLIC_FP32 = 0,           /* float in/out, fast-math solver                      */
-    PLIC_FP32_POLISHED = 1,  /* float in/out, solver + one Newton step on Eq. 10    */
+    PLIC_FP32_POLISHED = 1,  /* float in/out, solver + one Newton step on Eq. 10.  For
+                                the optimised SZ and the analytic solution (unless
+                                FAITHFUL) the two are one kernel, whose root ends with
+                                a Newton step either way                        */
     PLIC_FP64 = 2,           /* double in/out, the solver in double; plic_offset by
                                 the optimised SZ and the analytic solution (unless
                                 FAITHFUL) finishes an FP32 start by Newton steps in
                                 64-bit fixed point: |d0 error| below 2e-16 for
-                                |n| = 1                                         */
+                                |n| = 1 (4e-16 of the power of two above the largest
+                                component for normals of other lengths, which
+                                these two accept up to L = 3)                   */
     PLIC_FP64_REFINED = 3    /* double in/out.  plic_offset by the optimised SZ and the
                                 analytic solution: as PLIC_FP64.  By the others: the
                                 FP32 solver (polished) on the reduced problem, then

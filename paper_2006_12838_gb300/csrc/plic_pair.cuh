@@ -31,9 +31,6 @@ __device__ __forceinline__ b2 le(f2 a, f2 b) { return {a.x <= b.x, a.y <= b.y}; 
 
 __device__ __forceinline__ f2 rsqrt(f2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
 __device__ __forceinline__ f2 rcp(f2 a) { return make_float2(rcp_approx(a.x), rcp_approx(a.y)); }
-__device__ __forceinline__ f2 sqrt_(f2 a) {
-    return make_float2(Fm<float>::sqrt_(a.x), Fm<float>::sqrt_(a.y));
-}
 
 // cube root of x >= 0 as MUFU exp2(log2(x)/3): relative error below 6e-6
 // even for x = 1e-30 (the MUFU log2's absolute error, times |log2 x|/3), and
@@ -47,11 +44,10 @@ __device__ __forceinline__ f2 cbrt_(f2 x) {
                        Fm<float>::exp2f_approx(Fm<float>::__log2f_approx(x.y) * (1.0f / 3.0f)));
 }
 
-// sqrt of x >= 0 as x rsqrt(x) with 1e-30 added (no zero branch).  Both
-// callers pass arguments that are >= 0 wherever the result is used: the
-// arcsine's 1/2 (1 - a) with a <= 1, and the case-(2) radicand
-// 8 n2 n3 V - n1^2/3, which is >= n1^2 in case (2) and exactly 8 n2 n3 V >= 0
-// for n1 = 0.
+// sqrt of x >= 0 as x rsqrt(x) with 1e-30 added (no zero branch).  The callers
+// (centre_distance, sz_orig, and offset_two of the curvature step, which clamps it)
+// pass the case-(2) radicand 2 n2 n3 V - n1^2/12, which is >= n1^2/4 where the result is
+// used (6 n2 n3 V >= n1^2 there) and exactly 2 n2 n3 V >= 0 for n1 = 0.
 __device__ __forceinline__ f2 sqrtp(f2 x) {
     x = add(x, mk(1e-30f));
     return mul(x, rsqrt(x));

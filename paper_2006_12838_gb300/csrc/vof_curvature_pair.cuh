@@ -13,7 +13,8 @@ namespace plic {
 // root of the paired path); other methods solve one after the other.  These
 // solves are most of an interface cell's instructions, and the kernels are
 // issue bound: with the arcsine, the sine and a Newton step on Eq. 10 the batch of
-// 64 fields (2.59 M cells) took 252 us, with the root in units of t 207 us.
+// 64 fields (2.59 M cells) took 252 us, with a root of one polynomial and one step 207 us
+// (and 189 -> 191 with that step carried to the accuracy of the former, CentreRoot).
 template <int METHOD>
 __device__ __forceinline__ p2::f2 offset_two(const CellPlic<METHOD>& pl, p2::f2 V0) {
     return make_float2(pl.offset(V0.x), pl.offset(V0.y));
