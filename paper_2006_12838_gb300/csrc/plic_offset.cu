@@ -382,7 +382,7 @@ __device__ __noinline__ fx::u64 fx_rest(double nx, double ny, double nz, double 
 // every thread stores its own cells.  The arrays are read as integers: of the bits of a double in
 // a register the compiler makes |x| an operation on the FP64 pipe (three per cell:
 // 396 against 317 us).
-// Bound: instruction issue (477 warp instructions per 32 cells, 72 % of the slots; ALU
+// Bound: instruction issue (470 warp instructions per 32 cells, 71 % of the slots; ALU
 // pipe 68 % busy) beside the FP64 pipe (7 instructions, 67 %).  2^24 cells: closed forms 3200 us (optimised
 // SZ, FP64 pipe 85 % busy) and 4490 us (analytic); this scheme with one thread running
 // each of its cells through its case 379 us (every case of the warp in turn, 18.8 lanes
